@@ -427,6 +427,19 @@ static void derive_cst(const Phys &ph, double tol_floor, CstT<T> &c) {
   for (int r = 0; r < 4; ++r) c.kk[r] = T(ph.kessler_k[r]);
   c.kessler_tol = T(ph.kessler_tol > tol_floor ? ph.kessler_tol : tol_floor);
   c.c_vd = T(ph.c_vd);
+  const auto lo = [](double x) { return T(x - double(T(x))); };
+  c.c_vd_lo = lo(ph.c_vd);
+  c.R_d_lo = lo(ph.R_d);
+  for (int i = 0; i < kMaxVap; ++i) {
+    c.Tref[i] = T(ph.Tref[i]);
+    c.Tref_lo[i] = lo(ph.Tref[i]);
+    c.sig_v_lo[i] = lo(ph.sig_v[i]);
+    c.inv_eps_lo[i] = lo(ph.inv_eps[i]);
+    for (int j = 0; j < kMaxCond; ++j) {
+      c.sig_c_lo[i][j] = lo(ph.sig_c[i][j]);
+      c.mu_lo[i][j] = lo(ph.mu[i][j]);
+    }
+  }
   c.cool_rate = T(ph.cool_rate);
   c.cool_p_lo = T(ph.cool_p_lo);
   c.cool_p_hi = T(ph.cool_p_hi);
@@ -484,21 +497,91 @@ static int halos_ready(snap_ctx *ctx, const char *who) {
 static int apply_variant(snap_ctx *ctx, int v);
 static int build_class_tables(snap_ctx *ctx);
 
-// Default tile shape: the first variant (in the order built, the fastest on large grids) whose
-// tiles over all domains fill every SM at least once; else the one with the most tiles.
-static int default_variant(const snap_ctx *ctx) {
+// Multiprocessors of the current device (0 if it cannot be asked).
+static int device_sms() {
   int dev = 0, nsm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return 0;
+  return nsm;
+}
+
+// Tiles of the domains doms on a shape of tl[0] x tl[1] cells by cz levels.
+static long long count_tiles(const std::vector<DomDev> &doms, const int *tl, int cz) {
+  long long t = 0;
+  for (const DomDev &D : doms)
+    t += (long long)((D.nx + tl[0] - 1) / tl[0]) * ((D.ny + tl[1] - 1) / tl[1]) *
+         ((D.nz + cz - 1) / cz);
+  return t;
+}
+
+// Levels per tile of a marching shape, and what a stage costs with them in units of one level of
+// one tile on one SM: the busiest SM walks n = ceil(tiles / SMs) tiles of cz + 3 levels' work
+// (three levels' conversions and two z reconstructions go into the start of a tile). A tile alone
+// on its SM takes about 1.4 times its share of a full SM (its barriers and loads are not hidden
+// by another tile). Against a fixed 16 levels: the radiative-convective column 128 x 96 x 128
+// (288 tiles of 22 levels, two per SM at once, instead of 384) 1.33 -> 1.08 ms per step, dry 190 x
+// 131 x 85 (408 tiles of 22 levels instead of 612 of 16) 0.65 -> 0.47 ms.
+static int march_levels(const std::vector<DomDev> &doms, const TileVariant &tv, int nsm,
+                        double *cost) {
+  int nzmax = 0, best = tv.tile[2];
+  for (const DomDev &D : doms) nzmax = D.nz > nzmax ? D.nz : nzmax;
+  *cost = 1e300;
+  for (int cz = tv.tile[2]; cz >= 4; --cz) {
+    if (cz >= 2 * nzmax) continue;
+    const long long n = (count_tiles(doms, tv.tile, cz) + nsm - 1) / nsm;
+    const double c = (cz + 3) * (n == 1 ? 1.4 : double(n));
+    if (c < *cost) {
+      *cost = c;
+      best = cz;
+    }
+  }
+  return best;
+}
+
+// Divides the domains into the tiles of shape tv, numbered from 0; prefix receives the first
+// tile of each domain and the total.
+static void tile_domains(std::vector<DomDev> &doms, const TileVariant &tv, int *prefix) {
+  int cz = tv.tile[2];
+  if (tv.march) {
+    double cost;
+    const int nsm = device_sms();
+    cz = march_levels(doms, tv, nsm > 0 ? nsm : 1, &cost);
+  }
+  prefix[0] = 0;
+  for (size_t i = 0; i < doms.size(); ++i) {
+    DomDev &D = doms[i];
+    D.cz = cz;
+    D.tx = (D.nx + tv.tile[0] - 1) / tv.tile[0];
+    D.ty = (D.ny + tv.tile[1] - 1) / tv.tile[1];
+    D.tz = (D.nz + cz - 1) / cz;
+    D.tile_begin = prefix[i];
+    prefix[i + 1] = prefix[i] + D.tx * D.ty * D.tz;
+  }
+}
+
+// Default tile shape. A marching shape (first in its set) unless the grid is so small that the
+// one-shot tiles after it finish sooner: one such tile of 256 cells costs an SM 1.55 levels of a
+// marching tile (Jovian 8.6 against 5.5 us, dry 4.3 against 2.8), and no less than 2.4 when the
+// SM has only one or two. Else the first shape (in the order built, the fastest on large grids)
+// whose tiles over all domains fill every SM at least once; else the one with the most tiles.
+static int default_variant(const snap_ctx *ctx) {
+  const int nsm = device_sms();
+  if (nsm <= 0) return 0;
   int best = 0;
   long long best_tiles = -1;
   for (int v = 0; v < ctx->ks.nvariants; ++v) {
-    const int *tl = ctx->ks.var[v].tile;
-    long long t = 0;
-    for (const DomDev &D : ctx->dom)
-      t += (long long)((D.nx + tl[0] - 1) / tl[0]) * ((D.ny + tl[1] - 1) / tl[1]) *
-           ((D.nz + tl[2] - 1) / tl[2]);
+    const TileVariant &tv = ctx->ks.var[v];
+    if (tv.march) {
+      if (v + 1 == ctx->ks.nvariants) return v;
+      double cost;
+      march_levels(ctx->dom, tv, nsm, &cost);
+      const int *tl = ctx->ks.var[v + 1].tile;
+      const long long n = (count_tiles(ctx->dom, tl, tl[2]) + nsm - 1) / nsm;
+      if (cost <= std::max(1.55 * n, 2.4)) return v;
+      continue;
+    }
+    const long long t = count_tiles(ctx->dom, tv.tile, tv.tile[2]);
     if (t >= nsm) return v;
     if (t > best_tiles) {
       best_tiles = t;
@@ -575,17 +658,11 @@ extern "C" int snap_init_grid(snap_ctx **out, const snap_grid_desc *d, int n_dom
     ctx->ncells += (long long)nc;
     ctx->state_bytes += (long long)(nc * ctx->nv * ctx->word);
     nprof += 4 * (size_t)g.nz + 1;
-    nproff += 5 * (size_t)g.nz + 1;
+    nproff += 6 * (size_t)g.nz + 1;
     DomDev &D = ctx->dom[i];
     D.nx = g.nx;
     D.ny = g.ny;
     D.nz = g.nz;
-    const int *tl = ctx->ks.var[0].tile;
-    D.tx = (g.nx + tl[0] - 1) / tl[0];
-    D.ty = (g.ny + tl[1] - 1) / tl[1];
-    D.tz = (g.nz + tl[2] - 1) / tl[2];
-    D.tile_begin = ctx->prefix[i];
-    ctx->prefix[i + 1] = ctx->prefix[i] + D.tx * D.ty * D.tz;
     for (int s = 0; s < 6; ++s) D.bc[s] = g.bc[s];
     D.dx = g.dx;
     D.dy = g.ny > 1 ? g.dy : g.dx;
@@ -609,6 +686,7 @@ extern "C" int snap_init_grid(snap_ctx **out, const snap_grid_desc *d, int n_dom
       }
     }
   }
+  tile_domains(ctx->dom, ctx->ks.var[0], ctx->prefix.data());
   ctx->ntiles = ctx->prefix[n_domains];
   int ret = SNAP_OK;
   do {
@@ -675,7 +753,9 @@ extern "C" int snap_init_grid(snap_ctx **out, const snap_grid_desc *d, int n_dom
         proff[pof + k] = hi;
         proff[pof + g.nz + k] = (float)(g.rho_bar[k] - (double)hi);
         proff[pof + 2 * g.nz + k] = (float)prof[po + 2 * g.nz + 1 + k];
-        proff[pof + 4 * g.nz + 1 + k] = (float)prof[po + 3 * g.nz + 1 + k];
+        const double er_k = prof[po + 3 * g.nz + 1 + k];
+        proff[pof + 4 * g.nz + 1 + k] = (float)er_k;
+        proff[pof + 5 * g.nz + 1 + k] = (float)(er_k - (double)(float)er_k);
       }
       for (int k = 0; k <= g.nz; ++k) proff[pof + 3 * g.nz + k] = (float)g.p_bar_face[k];
       D.rb_hi = fb;
@@ -683,6 +763,7 @@ extern "C" int snap_init_grid(snap_ctx **out, const snap_grid_desc *d, int n_dom
       D.pc_f = fb + 2 * g.nz;
       D.pf_f = fb + 3 * g.nz;
       D.er_f = fb + 4 * g.nz + 1;
+      D.er_lo = fb + 5 * g.nz + 1;
       D.idx = 1.0 / D.dx;
       D.idy = 1.0 / D.dy;
       D.idz = 1.0 / D.dz;
@@ -694,7 +775,7 @@ extern "C" int snap_init_grid(snap_ctx **out, const snap_grid_desc *d, int n_dom
       D.rate_next = ctx->rate_next_dev + i;
       D.dt_step = ctx->dt_dev + i;
       po += 4 * (size_t)g.nz + 1;
-      pof += 5 * (size_t)g.nz + 1;
+      pof += 6 * (size_t)g.nz + 1;
     }
     if ((e = cudaMemcpy(ctx->prof_dev, prof.data(), sizeof(double) * nprof, cudaMemcpyHostToDevice)) != cudaSuccess) break;
     if ((e = cudaMemcpy(ctx->proff_dev, proff.data(), sizeof(float) * nproff, cudaMemcpyHostToDevice)) != cudaSuccess) break;
@@ -737,16 +818,7 @@ extern "C" int snap_init_grid(snap_ctx **out, const snap_grid_desc *d, int n_dom
 
 // Rebuild the tile tables of every domain for tile variant v and upload them.
 static int apply_variant(snap_ctx *ctx, int v) {
-  const int *tl = ctx->ks.var[v].tile;
-  ctx->prefix[0] = 0;
-  for (int i = 0; i < ctx->ndom; ++i) {
-    DomDev &D = ctx->dom[i];
-    D.tx = (D.nx + tl[0] - 1) / tl[0];
-    D.ty = (D.ny + tl[1] - 1) / tl[1];
-    D.tz = (D.nz + tl[2] - 1) / tl[2];
-    D.tile_begin = ctx->prefix[i];
-    ctx->prefix[i + 1] = ctx->prefix[i] + D.tx * D.ty * D.tz;
-  }
+  tile_domains(ctx->dom, ctx->ks.var[v], ctx->prefix.data());
   ctx->ntiles = ctx->prefix[ctx->ndom];
   ctx->grid = ctx->ntiles;
   const int mrb = ctx->ks.var[v].max_resident_blocks();
@@ -860,21 +932,14 @@ static int build_class_tables(snap_ctx *ctx) {
   ctx->cls_prefix.clear();
   ctx->cls_off.assign(nc, 0);
   for (int c = 0; c < nc; ++c) {
-    const int *tl = ctx->ks.var[ctx->cls_tv[c]].tile;
     ctx->cls_off[c] = (int)ctx->cls_dom.size();
-    int t = 0;
-    ctx->cls_prefix.push_back(0);
-    for (int i : ctx->cls[c]) {
-      DomDev D = ctx->dom[i];
-      D.tx = (D.nx + tl[0] - 1) / tl[0];
-      D.ty = (D.ny + tl[1] - 1) / tl[1];
-      D.tz = (D.nz + tl[2] - 1) / tl[2];
-      D.tile_begin = t;
-      t += D.tx * D.ty * D.tz;
-      ctx->cls_dom.push_back(D);
-      ctx->cls_prefix.push_back(t);
-    }
-    ctx->cls_ntiles[c] = t;
+    std::vector<DomDev> doms;
+    for (int i : ctx->cls[c]) doms.push_back(ctx->dom[i]);
+    std::vector<int> prefix(doms.size() + 1);
+    tile_domains(doms, ctx->ks.var[ctx->cls_tv[c]], prefix.data());
+    ctx->cls_dom.insert(ctx->cls_dom.end(), doms.begin(), doms.end());
+    ctx->cls_prefix.insert(ctx->cls_prefix.end(), prefix.begin(), prefix.end());
+    ctx->cls_ntiles[c] = prefix.back();
   }
   if (!ctx->cls_doms_dev) {
     CK(cudaMalloc(&ctx->cls_doms_dev, sizeof(DomDev) * ctx->ndom));
@@ -964,11 +1029,12 @@ static bool resident_possible(snap_ctx *ctx, std::string *why) {
 static int build_resident(snap_ctx *ctx) {
   std::string why;
   if (!resident_possible(ctx, &why)) return fail(ctx, SNAP_ENOTSUP, "snap_use_persistent: " + why);
-  const int *tl = ctx->ks.var[ctx->tv].tile;
+  const int *shape = ctx->ks.var[ctx->tv].tile;
   const int nt = ctx->ntiles;
   std::vector<std::vector<int>> dep(nt);
   for (int i = 0; i < ctx->ndom; ++i) {
     const DomDev &D = ctx->dom[i];
+    const int tl[3] = {shape[0], shape[1], D.cz};
     const int n[3] = {D.nx, D.ny, D.nz}, tc[3] = {D.tx, D.ty, D.tz};
     const bool per[3] = {D.bc[0] == kBcPeriodic, D.bc[2] == kBcPeriodic, false};
     for (int t = 0; t < tc[0] * tc[1] * tc[2]; ++t) {
@@ -1578,8 +1644,10 @@ extern "C" int snap_get_class_info(const snap_ctx *ctx, int cls, int *n_domains,
   const DomDev &D = ctx->dom[ctx->cls[cls][0]];
   if (n_domains) *n_domains = (int)ctx->cls[cls].size();
   if (cells) *cells = D.nx * D.ny * D.nz;
-  if (tile)
-    for (int i = 0; i < 3; ++i) tile[i] = ctx->ks.var[v].tile[i];
+  if (tile) {
+    for (int i = 0; i < 2; ++i) tile[i] = ctx->ks.var[v].tile[i];
+    tile[2] = ctx->per_class ? ctx->cls_dom[ctx->cls_off[cls]].cz : D.cz;
+  }
   if (variant) *variant = v;
   return SNAP_OK;
 }
@@ -1753,7 +1821,8 @@ extern "C" int snap_get_info(const snap_ctx *ctx, snap_info *info) {
   info->nfields = ctx->nv;
   info->ncells_total = ctx->ncells;
   info->state_bytes = ctx->state_bytes;
-  for (int i = 0; i < 3; ++i) info->tile[i] = ctx->ks.var[ctx->tv].tile[i];
+  for (int i = 0; i < 2; ++i) info->tile[i] = ctx->ks.var[ctx->tv].tile[i];
+  info->tile[2] = ctx->dom[0].cz;
   info->tiles_total = ctx->ntiles;
   info->kernel_launches_per_step = ctx->persistent ? 1 : 3;
   info->tile_variant = ctx->tv;

@@ -1,5 +1,5 @@
 // kern_moist3d.cu -- stage kernels for two vapours with cloud and precipitation, 3-D.
-#include "snap_stage.cuh"
+#include "snap_march.cuh"
 
 namespace snap {
 
@@ -10,11 +10,14 @@ bool find_kernels_moist3d(int f32, int visc, int micro, KernelSet *out) {
   using A = TileT<8, 8, 4, 256, 3>;
   using A64 = TileT<8, 8, 4>;
   using B = TileT<16, 8, 2, 256, 2>;
+  // the march along z first (its shared memory allows 2 CTAs per SM in FP32, 1 in FP64)
+  using M = MarchT<32, 8, 32, 2>;
+  using M64 = MarchT<32, 8, 32, 1>;
   if (visc) return false;
   if (micro)  // sedimentation and the Kessler scheme compiled in, default tile only
-    *out = f32 ? Family<float, L>::set_micro<A>() : Family<double, L>::set_micro<A64>();
+    *out = f32 ? Family<float, L>::set_micro<M, A>() : Family<double, L>::set_micro<M64, A64>();
   else
-    *out = f32 ? Family<float, L>::set<false, A, B>() : Family<double, L>::set<false, A64>();
+    *out = f32 ? Family<float, L>::set<false, M, A, B>() : Family<double, L>::set<false, M64, A64>();
   return true;
 }
 

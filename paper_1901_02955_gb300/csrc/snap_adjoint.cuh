@@ -922,13 +922,13 @@ __global__ void __launch_bounds__(128) adj_cell_kernel(const AdjArgs a) {
 // |u|^2/2 (other condensates). lam (in place): (dY_out/dY_in)^T lam.
 template <class R, class L>
 __device__ __forceinline__ void satadj_adj_cell(const Phys &ph, const CstT<R> &C, const R *y,
-                                                double eref, R *lam) {
+                                                typename Wide<R>::T eref, R *lam) {
   constexpr int NV = L::NV, IM0 = L::IM0;
-  // T from the conserved energy in FP64 (the inversion cancels large terms); the derivative
-  // itself in the kernel's type
-  double Td, pd;
-  cell_Tp<R, L>(ph, y, eref, Td, pd);
-  const R T = R(Td), cvd = C.R_d * C.igm1;
+  // T from the conserved energy in wide numbers (the inversion cancels large terms); the
+  // derivative itself in the kernel's type
+  typename Wide<R>::T Tw, Cvw, Rmw;
+  invert_T<R, L>(ph, C, y, eref, Tw, Cvw, Rmw);
+  const R T = Wide<R>::r(Tw), cvd = C.R_d * C.igm1;
   R rho = R(0), u2 = R(0), Cv = y[0];
 #pragma unroll
   for (int s = 0; s < IM0; ++s) rho += y[s];
@@ -991,7 +991,7 @@ __global__ void __launch_bounds__(128) adj_satadj_kernel(const AdjArgs a) {
       y[v] = Yo[v * ncell + c];
       l[v] = lam[v * ncell + c];
     }
-    satadj_adj_cell<R, L>(a.ph, acst<R>(a), y, D.e_ref[c / plane], l);
+    satadj_adj_cell<R, L>(a.ph, acst<R>(a), y, Wide<R>::e_ref(D, int(c / plane)), l);
 #pragma unroll
     for (int v = 0; v < L::NV; ++v) lam[v * ncell + c] = l[v];
   }

@@ -43,6 +43,11 @@ struct CstT {
   T sig_c[kMaxVap][kMaxCond], sigc_m1[kMaxVap][kMaxCond], mu[kMaxVap][kMaxCond];
   T pref[kMaxVap], beta[kMaxVap], delta[kMaxVap], inv_Tref[kMaxVap], sighat_m1[kMaxVap];
   T w_term[kMaxCond], kk[4], kessler_tol, c_vd;
+  T Tref[kMaxVap];
+  // what the FP64 constant holds beyond its rounding to T (FP32 kernels carry the temperature
+  // inversion in pairs of floats)
+  T sig_v_lo[kMaxVap], sig_c_lo[kMaxVap][kMaxCond], inv_eps_lo[kMaxVap], mu_lo[kMaxVap][kMaxCond];
+  T Tref_lo[kMaxVap], c_vd_lo, R_d_lo;
   T cool_rate, cool_p_lo, cool_p_hi, sponge_itau0, sponge_ip0;
 };
 
@@ -54,6 +59,7 @@ struct DomDev {
   int nx, ny, nz;
   int tx, ty, tz;            // tiles per direction
   int tile_begin;            // first tile index of this domain in the launch
+  int cz;                    // levels per tile
   int bc[6];
   double dx, dy, dz;
   double grav, cfl, dt_fixed;
@@ -70,6 +76,7 @@ struct DomDev {
   const float *pc_f;         // [nz]
   const float *pf_f;         // [nz+1]
   const float *er_f;         // [nz]
+  const float *er_lo;        // [nz] e_ref - er_f
   double idx, idy, idz;      // inverse cell sizes
   float fidx, fidy, fidz, fgrav;
   unsigned long long *rate;  // CFL rate max as double bits (non-negative doubles order as
@@ -127,7 +134,8 @@ enum Flag : unsigned int { kFlagNonFinite = 1u, kFlagNoConv = 2u, kFlagTimeout =
 
 // One tile shape of a kernel family.
 struct TileVariant {
-  int tile[3];
+  int tile[3];               // march: tile[2] is the most levels a tile may have
+  int march;                 // 1: walked level by level (snap_march.cuh)
   int threads;
   size_t smem_stage;
   cudaError_t (*stage)(const StageArgs &, int grid, cudaStream_t);

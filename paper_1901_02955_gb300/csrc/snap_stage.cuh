@@ -131,6 +131,14 @@ __device__ __forceinline__ const CstT<double> &cst<double>(const StageArgs &a) {
 template <int TX_, int TY_, int TZ_, int NT_ = 256, int MINB_ = 0>
 struct TileT {
   static constexpr int TX = TX_, TY = TY_, TZ = TZ_, NT = NT_, MINB = MINB_;
+  static constexpr bool MARCH = false;
+};
+// A tile of TX x TY columns of at most TZ levels (DomDev::cz of them) walked level by level, one
+// thread per column (snap_march.cuh).
+template <int TX_, int TY_, int TZ_, int MINB_ = 0>
+struct MarchT {
+  static constexpr int TX = TX_, TY = TY_, TZ = TZ_, NT = TX_ * TY_, MINB = MINB_;
+  static constexpr bool MARCH = true;
 };
 
 template <class T, bool D3>
@@ -246,43 +254,53 @@ struct SV {
 };
 
 // Per-level reference values in the kernel's type: FP32 kernels read FP32 copies, FP64
-// kernels the FP64 originals.
+// kernels the FP64 originals. DD is DomDev, or a kernel's own copy of what it needs of it.
 template <class R>
 struct Prof;
 template <>
 struct Prof<float> {
-  static __device__ __forceinline__ float pc(const DomDev &D, int k) { return D.pc_f[k]; }
-  static __device__ __forceinline__ float pf(const DomDev &D, int k) { return D.pf_f[k]; }
-  static __device__ __forceinline__ float er(const DomDev &D, int k) { return D.er_f[k]; }
+  template <class DD>
+  static __device__ __forceinline__ float pc(const DD &D, int k) { return D.pc_f[k]; }
+  template <class DD>
+  static __device__ __forceinline__ float pf(const DD &D, int k) { return D.pf_f[k]; }
+  template <class DD>
+  static __device__ __forceinline__ float er(const DD &D, int k) { return D.er_f[k]; }
   // rho - rho_bar_k from the conserved densities y: dry air minus the FP32 head of rho_bar is
   // exact (the two are within a factor of 2), the tracers are added to that small difference,
   // and the FP32 tail of rho_bar (rb_lo) last
-  template <class L>
-  static __device__ __forceinline__ float drho(const DomDev &D, int k, const float *y) {
+  template <class L, class DD>
+  static __device__ __forceinline__ float drho(const DD &D, int k, const float *y) {
     float r = y[0] - D.rb_hi[k];
 #pragma unroll
     for (int s = 1; s < L::IM0; ++s) r += y[s];
     return r - D.rb_lo[k];
   }
-  static __device__ __forceinline__ float grav(const DomDev &D) { return D.fgrav; }
-  static __device__ __forceinline__ float ih(const DomDev &D, int d) {
+  template <class DD>
+  static __device__ __forceinline__ float grav(const DD &D) { return D.fgrav; }
+  template <class DD>
+  static __device__ __forceinline__ float ih(const DD &D, int d) {
     return d == 0 ? D.fidx : (d == 1 ? D.fidy : D.fidz);
   }
 };
 template <>
 struct Prof<double> {
-  static __device__ __forceinline__ double pc(const DomDev &D, int k) { return D.p_cell[k]; }
-  static __device__ __forceinline__ double pf(const DomDev &D, int k) { return D.p_face[k]; }
-  static __device__ __forceinline__ double er(const DomDev &D, int k) { return D.e_ref[k]; }
-  template <class L>
-  static __device__ __forceinline__ double drho(const DomDev &D, int k, const double *y) {
+  template <class DD>
+  static __device__ __forceinline__ double pc(const DD &D, int k) { return D.p_cell[k]; }
+  template <class DD>
+  static __device__ __forceinline__ double pf(const DD &D, int k) { return D.p_face[k]; }
+  template <class DD>
+  static __device__ __forceinline__ double er(const DD &D, int k) { return D.e_ref[k]; }
+  template <class L, class DD>
+  static __device__ __forceinline__ double drho(const DD &D, int k, const double *y) {
     double r = y[0];
 #pragma unroll
     for (int s = 1; s < L::IM0; ++s) r += y[s];
     return r - D.rho_bar[k];
   }
-  static __device__ __forceinline__ double grav(const DomDev &D) { return D.grav; }
-  static __device__ __forceinline__ double ih(const DomDev &D, int d) {
+  template <class DD>
+  static __device__ __forceinline__ double grav(const DD &D) { return D.grav; }
+  template <class DD>
+  static __device__ __forceinline__ double ih(const DD &D, int d) {
     return d == 0 ? D.idx : (d == 1 ? D.idy : D.idz);
   }
 };
@@ -295,8 +313,8 @@ struct Prof<double> {
 // pressure is returned in p_tot and T in T_out. Dry: p - pbar = (gamma_d - 1)(y_E - K) is
 // formed from small numbers. Moist: the inversion U = rho e - K - A, T = U / C_v, p = R_m T
 // runs in FP64.
-template <class R, class L>
-__device__ __forceinline__ void cons_to_prim(const Phys &ph, const CstT<R> &C, const DomDev &D,
+template <class R, class L, class DD>
+__device__ __forceinline__ void cons_to_prim(const Phys &ph, const CstT<R> &C, const DD &D,
                                              int k, const R *y, R *x, R &p_tot, R &T_out) {
   R rho = y[0];
 #pragma unroll
@@ -450,79 +468,222 @@ __device__ __forceinline__ void lmars(const CstT<R> &C, const R *XL, const R *XR
 }
 
 // ------------------------------------------------------------------------------------------
+// The temperature inversion's wide numbers: the energy U, the heat capacity, the gas sum and T
+// need more digits than FP32 holds (T - T^r decides the saturation pressure, U carries the
+// kinetic and latent energies as small differences). FP64 kernels use FP64. FP32 kernels use an
+// unevaluated pair h + l of floats (|l| <= ulp(h) / 2, about 48 bits), from the error-free sum
+// and product of Knuth and Dekker (the product by a fused multiply-add): on this part an FP64
+// instruction holds its pipe 64 cycles per warp, a pair operation is 6 to 12 FP32 instructions.
+// A quotient of pairs is good to ~1e-13, where the FP64 form it replaces (one Newton-Raphson
+// step) had ~1e-12; sums and products to ~1e-14. Error against FP64 of the adjusted state over
+// Jovian and Earth cells: unchanged (below the state's own FP32 rounding).
+// ------------------------------------------------------------------------------------------
+struct Df {
+  float h, l;
+};
+__device__ __forceinline__ Df quick2(float a, float b) {  // |a| >= |b|
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ Df sum2(float a, float b) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Df operator+(Df a, float b) {
+  const Df s = sum2(a.h, b);
+  return quick2(s.h, __fadd_rn(s.l, a.l));
+}
+__device__ __forceinline__ Df operator+(Df a, Df b) {
+  const Df s = sum2(a.h, b.h);
+  return quick2(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ Df operator-(Df a, Df b) { return a + Df{-b.h, -b.l}; }
+__device__ __forceinline__ Df operator*(Df a, float b) {
+  const float p = __fmul_rn(a.h, b);
+  return quick2(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+}
+__device__ __forceinline__ Df operator*(Df a, Df b) {
+  const float p = __fmul_rn(a.h, b.h);
+  return quick2(p, __fmaf_rn(a.h, b.l, __fmaf_rn(a.l, b.h, __fmaf_rn(a.h, b.h, -p))));
+}
+// a / b: the approximate quotient q of the heads, then the remainder a - q b over b
+__device__ __forceinline__ Df operator/(Df a, Df b) {
+  const float r = Ar<float>::rcp(b.h), q = __fmul_rn(a.h, r);
+  const float e = __fadd_rn(__fmaf_rn(-q, b.h, a.h), __fmaf_rn(-q, b.l, a.l));
+  return quick2(q, __fmul_rn(e, r));
+}
+
+template <class R>
+struct Wide;
+template <>
+struct Wide<float> {
+  using T = Df;
+  static __device__ __forceinline__ T of(float x) { return {x, 0.0f}; }
+  static __device__ __forceinline__ float r(T x) { return x.h; }
+  static __device__ __forceinline__ T diff(float a, float b) { return sum2(a, -b); }
+  template <class DD>
+  static __device__ __forceinline__ T e_ref(const DD &D, int k) { return {D.er_f[k], D.er_lo[k]}; }
+  static __device__ __forceinline__ T c_vd(const Phys &, const CstT<float> &C) { return {C.c_vd, C.c_vd_lo}; }
+  static __device__ __forceinline__ T R_d(const Phys &, const CstT<float> &C) { return {C.R_d, C.R_d_lo}; }
+  static __device__ __forceinline__ T Tref(const Phys &, const CstT<float> &C, int i) { return {C.Tref[i], C.Tref_lo[i]}; }
+  static __device__ __forceinline__ T sig_v(const Phys &, const CstT<float> &C, int i) { return {C.sig_v[i], C.sig_v_lo[i]}; }
+  static __device__ __forceinline__ T sig_c(const Phys &, const CstT<float> &C, int i, int j) { return {C.sig_c[i][j], C.sig_c_lo[i][j]}; }
+  static __device__ __forceinline__ T inv_eps(const Phys &, const CstT<float> &C, int i) { return {C.inv_eps[i], C.inv_eps_lo[i]}; }
+  static __device__ __forceinline__ T mu(const Phys &, const CstT<float> &C, int i, int j) { return {C.mu[i][j], C.mu_lo[i][j]}; }
+  static __device__ __forceinline__ T quot(T a, T b) { return a / b; }
+};
+template <>
+struct Wide<double> {
+  using T = double;
+  static __device__ __forceinline__ T of(double x) { return x; }
+  static __device__ __forceinline__ double r(T x) { return x; }
+  static __device__ __forceinline__ T diff(double a, double b) { return a - b; }
+  template <class DD>
+  static __device__ __forceinline__ T e_ref(const DD &D, int k) { return D.e_ref[k]; }
+  static __device__ __forceinline__ T c_vd(const Phys &ph, const CstT<double> &) { return ph.c_vd; }
+  static __device__ __forceinline__ T R_d(const Phys &ph, const CstT<double> &) { return ph.R_d; }
+  static __device__ __forceinline__ T Tref(const Phys &ph, const CstT<double> &, int i) { return ph.Tref[i]; }
+  static __device__ __forceinline__ T sig_v(const Phys &ph, const CstT<double> &, int i) { return ph.sig_v[i]; }
+  static __device__ __forceinline__ T sig_c(const Phys &ph, const CstT<double> &, int i, int j) { return ph.sig_c[i][j]; }
+  static __device__ __forceinline__ T inv_eps(const Phys &ph, const CstT<double> &, int i) { return ph.inv_eps[i]; }
+  static __device__ __forceinline__ T mu(const Phys &ph, const CstT<double> &, int i, int j) { return ph.mu[i][j]; }
+  static __device__ __forceinline__ T quot(T a, T b) { return Ar<double>::div(a, b); }
+};
+
+// T, the heat capacity at constant volume (J/(m^3 K)) and the sum of the gas densities over
+// their molar-mass ratios, from the stored conserved values y (energy as rho e - eref): U =
+// rho e - K - A, T = U / C_v (Eq. energy, App. B). The FP32 kernels sum the kinetic and latent
+// energies (about 1e-4 of U) and the density they need in FP32: their rounding is ~1e-10 of U.
+template <class R, class L>
+__device__ __forceinline__ void invert_T(const Phys &ph, const CstT<R> &C, const R *y,
+                                         typename Wide<R>::T eref, typename Wide<R>::T &T,
+                                         typename Wide<R>::T &Cv, typename Wide<R>::T &Rm) {
+  using W = Wide<R>;
+  Cv = W::of(y[0]);
+  Rm = W::of(y[0]);
+#pragma unroll
+  for (int i = 0; i < L::NVAP; ++i) {
+    Cv = Cv + W::sig_v(ph, C, i) * y[1 + i];
+    Rm = Rm + W::inv_eps(ph, C, i) * y[1 + i];
+#pragma unroll
+    for (int j = 0; j < L::NCOND; ++j) Cv = Cv + W::sig_c(ph, C, i, j) * y[L::cond(i, j)];
+  }
+  R rho = y[0], K2 = R(0), A = R(0);
+#pragma unroll
+  for (int s = 1; s < L::IM0; ++s) rho += y[s];
+#pragma unroll
+  for (int m = 0; m < L::NMOM; ++m) K2 = Ar<R>::fma_(y[L::IM0 + m], y[L::IM0 + m], K2);
+#pragma unroll
+  for (int i = 0; i < L::NVAP; ++i)
+#pragma unroll
+    for (int j = 0; j < L::NCOND; ++j) A = Ar<R>::fma_(C.mu[i][j], y[L::cond(i, j)], A);
+  Cv = Cv * W::c_vd(ph, C);
+  if constexpr (sizeof(R) == 4)
+    T = W::quot((eref + y[L::IE]) + -(R(0.5) * K2 * Ar<R>::rcp(rho) + A), Cv);
+  else
+    T = W::quot((eref + y[L::IE]) - R(0.5) * K2 * Ar<R>::rcp(rho) - A, Cv);
+}
+
+// ------------------------------------------------------------------------------------------
 // App. D saturation adjustment of one cell (isochoric). Each sweep visits the vapours in
 // order: projected molar transfer of Eq. dxf with the isochoric alpha, limited to keep both
 // phases non-negative, then T and p follow from the conserved energy and the equation of
 // state. Returns the sweep count, or -1 without convergence.
 // ------------------------------------------------------------------------------------------
-// An FP64 quotient a / b for the kernels of type R: FP64 kernels to about an ulp (two
-// Newton-Raphson steps, Ar<double>::div); FP32 kernels, whose states hold 7 digits, to ~1e-12
-// (one step from the approximate FP64 reciprocal)
-template <class R>
-__device__ __forceinline__ double quot64(double a, double b) {
-  if constexpr (sizeof(R) == 8) {
-    return Ar<double>::div(a, b);
-  } else {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(b));
-    r = fma(r, fma(-b, r, 1.0), r);
-    return a * r;
-  }
-}
-
+// The sweeps of one cell, from the inversion on.
 template <class R, class L>
-__device__ __forceinline__ void cell_Tp(const Phys &ph, const R *y, double eref, double &T,
-                                        double &p, double *Cv_out = nullptr,
-                                        double *Rm_out = nullptr) {
-  double Cv = y[0], Rm = y[0];
+__device__ __forceinline__ int satadj_sweeps(const Phys &ph, const CstT<R> &C, R *y,
+                                             typename Wide<R>::T eref, int max_iter) {
+  // T from the conserved energy once, in wide numbers (Eq. energy, App. B); after each transfer
+  // it is carried forward by the change of the two densities: rho e and the momenta are
+  // fixed, so C_v T + A is, and T' = T - (dA + T dC) / (C_v + dC), p' = R_d (R_m + dR_m) T'
+  // -- exact algebra, no inversion per sweep
+  using W = Wide<R>;
+  typename W::T Tw, Cvw, Rmw;
+  invert_T<R, L>(ph, C, y, eref, Tw, Cvw, Rmw);
+  R p = W::r(Rmw * W::R_d(ph, C) * Tw);
+  for (int sweep = 1; sweep <= max_iter; ++sweep) {
+    bool conv = true;
 #pragma unroll
-  for (int i = 0; i < L::NVAP; ++i) {
-    Cv += ph.sig_v[i] * double(y[1 + i]);
-    Rm += ph.inv_eps[i] * double(y[1 + i]);
+    for (int i = 0; i < L::NVAP; ++i) {
+      R T = W::r(Tw);
+      const R dTr = W::r(Tw - W::Tref(ph, C, i));  // T - T^r kept accurate: s(T) is steep
+      R N = y[0], gas = y[0], heat = R(0);
 #pragma unroll
-    for (int j = 0; j < L::NCOND; ++j) Cv += ph.sig_c[i][j] * double(y[L::cond(i, j)]);
+      for (int k = 0; k < L::NVAP; ++k) {
+        R tot = y[1 + k];
+#pragma unroll
+        for (int j = 0; j < L::NCOND; ++j) tot += y[L::cond(k, j)];
+        N += tot * C.inv_eps[k];
+        gas += y[1 + k] * C.inv_eps[k];
+        heat += tot * C.inv_eps[k] * C.sighat_m1[k];
+      }
+      const R iN = Ar<R>::rcp(N);
+      heat *= iN;
+      R qv = y[1 + i] * C.inv_eps[i] * iN;
+      R qc = y[L::cond(i, 0)] * C.inv_eps[i] * iN;
+      R gsum = gas * iN - qv;
+      R t = T * C.inv_Tref[i];
+      // p* = p^r exp[beta (1 - 1/t) - delta ln t] with 1 - 1/t = (T - T^r) / T
+      const R arg = C.beta[i] * dTr * Ar<R>::rcp(T) - C.delta[i] * Ar<R>::log_(t);
+      R ps = C.pref[i] * Ar<R>::exp_(arg);
+      // the arithmetic type holds p* only to ~(|arg| + 2) eps relative (the exponent's own
+      // rounding), so the transfer cannot settle below that: the stop test allows 4 times it
+      const R tol = fmax(C.satadj_tol, R(4) * (fabs(arg) + R(2)) * R(Ar<R>::eps));
+      R s = Ar<R>::div(ps, p);
+      R dq;
+      if (s >= R(1)) {
+        dq = -qc;
+      } else {
+        R bt = C.beta[i] * Ar<R>::rcp(t) - C.delta[i];
+        R alpha = C.gm1 * (bt - R(1)) * Ar<R>::rcp(R(1) + heat);
+        R om = R(1) - s;
+        R r = Ar<R>::div(s, om);
+        dq = Ar<R>::div(qv - r * gsum, R(1) + Ar<R>::div(s, om * om) * bt * alpha * gsum);
+      }
+      R drho;
+      if (dq >= qv) {
+        dq = qv;
+        drho = y[1 + i];
+      } else if (dq <= -qc) {
+        dq = -qc;
+        drho = -y[L::cond(i, 0)];
+      } else {
+        drho = dq * C.eps[i] * N;
+      }
+      if (drho != R(0)) {
+        const R yv = y[1 + i], yc = y[L::cond(i, 0)];
+        y[1 + i] -= drho;
+        y[L::cond(i, 0)] += drho;
+        // the changes as stored (after rounding to the state's type)
+        if constexpr (sizeof(R) == 4) {
+          // FP32 states: the increments in FP32 (good to ~1e-7 of themselves, ~1e-10 of T),
+          // accumulated into the wide T, heat capacity and gas sum
+          const R dv = y[1 + i] - yv, dc = y[L::cond(i, 0)] - yc;
+          const R dC = (C.sig_v[i] * dv + C.sig_c[i][0] * dc) * C.c_vd;
+          const R dT = (C.mu[i][0] * dc + T * dC) * Ar<R>::rcp(W::r(Cvw) + dC);
+          Tw = Tw + -dT;
+          Cvw = Cvw + dC;
+          Rmw = Rmw + C.inv_eps[i] * dv;
+        } else {
+          const double dv = double(y[1 + i]) - double(yv);
+          const double dc = double(y[L::cond(i, 0)]) - double(yc);
+          const double dC = (ph.sig_v[i] * dv + ph.sig_c[i][0] * dc) * ph.c_vd;
+          Tw -= Ar<double>::div(ph.mu[i][0] * dc + Tw * dC, Cvw + dC);
+          Cvw += dC;
+          Rmw += ph.inv_eps[i] * dv;
+        }
+        p = W::r(Rmw * W::R_d(ph, C) * Tw);
+      }
+      if (fabs(dq) > tol * (qv + qc)) conv = false;
+    }
+    if (conv) return sweep;
   }
-  double U;
-  if constexpr (sizeof(R) == 4) {
-    // FP32 states: the kinetic and latent energies (about 1e-4 of U) and the density they
-    // need are summed in FP32 -- their rounding is ~1e-10 of U, far below what the state holds
-    // -- and the inversion itself (U, the heat capacity, T, p) stays in FP64 with a quotient
-    // good to ~1e-12 (one Newton-Raphson step from the approximate FP64 reciprocal); an FP64
-    // instruction costs ~32 FP32 ones on this part
-    float rho = y[0], K2 = 0.0f, A = 0.0f;
-#pragma unroll
-    for (int s = 1; s < L::IM0; ++s) rho += y[s];
-#pragma unroll
-    for (int m = 0; m < L::NMOM; ++m) K2 = fmaf(y[L::IM0 + m], y[L::IM0 + m], K2);
-#pragma unroll
-    for (int i = 0; i < L::NVAP; ++i)
-#pragma unroll
-      for (int j = 0; j < L::NCOND; ++j) A = fmaf(float(ph.mu[i][j]), y[L::cond(i, j)], A);
-    U = (double(y[L::IE]) + eref) - double(0.5f * K2 * Ar<float>::rcp(rho) + A);
-    T = quot64<R>(U, Cv * ph.c_vd);
-  } else {
-    double rho = 0.0, K2 = 0.0, A = 0.0;
-#pragma unroll
-    for (int s = 0; s < L::IM0; ++s) rho += double(y[s]);
-#pragma unroll
-    for (int m = 0; m < L::NMOM; ++m) K2 += double(y[L::IM0 + m]) * double(y[L::IM0 + m]);
-#pragma unroll
-    for (int i = 0; i < L::NVAP; ++i)
-#pragma unroll
-      for (int j = 0; j < L::NCOND; ++j) A += ph.mu[i][j] * double(y[L::cond(i, j)]);
-    // quotients by the Newton-Raphson reciprocal of Ar<double> (within about an ulp of the
-    // IEEE quotient, a third of its FP64 instructions)
-    U = (double(y[L::IE]) + eref) - 0.5 * K2 * Ar<double>::rcp(rho) - A;
-    T = Ar<double>::div(U, Cv * ph.c_vd);
-  }
-  p = Rm * ph.R_d * T;
-  if (Cv_out) *Cv_out = Cv * ph.c_vd;  // heat capacity at constant volume, J/(m^3 K)
-  if (Rm_out) *Rm_out = Rm;            // sum of the gas densities / molar-mass ratios
+  return -1;
 }
-
 template <class R, class L>
-__device__ int satadj_cell(const Phys &ph, const CstT<R> &C, R *y, double eref, R eref_r,
-                           int max_iter) {
+__device__ __forceinline__ int satadj_cell(const Phys &ph, const CstT<R> &C, R *y, typename Wide<R>::T eref,
+                           R eref_r, int max_iter) {
   if constexpr (!L::MOIST) {
     return 0;
   } else {
@@ -563,90 +724,7 @@ __device__ int satadj_cell(const Phys &ph, const CstT<R> &C, R *y, double eref, 
         if (clear) return 1;
       }
     }
-    // T and p from the conserved energy once, in FP64 (Eq. energy, App. B); after each
-    // transfer they are carried forward in FP64 by the change of the two densities: rho e
-    // and the momenta are fixed, so C_v T + A is, and T' = T - (dA + T dC) / (C_v + dC),
-    // p' = R_d (R_m + dR_m) T' -- exact algebra, no inversion per sweep
-    double Td = 0.0, pd = 0.0, Cvd = 0.0, Rmd = 0.0;
-    cell_Tp<R, L>(ph, y, eref, Td, pd, &Cvd, &Rmd);
-    for (int sweep = 1; sweep <= max_iter; ++sweep) {
-      bool conv = true;
-#pragma unroll
-      for (int i = 0; i < L::NVAP; ++i) {
-        R T = R(Td), p = R(pd);
-        const R dTr = R(Td - ph.Tref[i]);  // T - T^r kept accurate: s(T) is steep
-        R N = y[0], gas = y[0], heat = R(0);
-#pragma unroll
-        for (int k = 0; k < L::NVAP; ++k) {
-          R tot = y[1 + k];
-#pragma unroll
-          for (int j = 0; j < L::NCOND; ++j) tot += y[L::cond(k, j)];
-          N += tot * C.inv_eps[k];
-          gas += y[1 + k] * C.inv_eps[k];
-          heat += tot * C.inv_eps[k] * C.sighat_m1[k];
-        }
-        const R iN = Ar<R>::rcp(N);
-        heat *= iN;
-        R qv = y[1 + i] * C.inv_eps[i] * iN;
-        R qc = y[L::cond(i, 0)] * C.inv_eps[i] * iN;
-        R gsum = gas * iN - qv;
-        R t = T * C.inv_Tref[i];
-        // p* = p^r exp[beta (1 - 1/t) - delta ln t] with 1 - 1/t = (T - T^r) / T
-        const R arg = C.beta[i] * dTr * Ar<R>::rcp(T) - C.delta[i] * Ar<R>::log_(t);
-        R ps = C.pref[i] * Ar<R>::exp_(arg);
-        // the arithmetic type holds p* only to ~(|arg| + 2) eps relative (the exponent's own
-        // rounding), so the transfer cannot settle below that: the stop test allows 4 times it
-        const R tol = fmax(C.satadj_tol, R(4) * (fabs(arg) + R(2)) * R(Ar<R>::eps));
-        R s = Ar<R>::div(ps, p);
-        R dq;
-        if (s >= R(1)) {
-          dq = -qc;
-        } else {
-          R bt = C.beta[i] * Ar<R>::rcp(t) - C.delta[i];
-          R alpha = C.gm1 * (bt - R(1)) * Ar<R>::rcp(R(1) + heat);
-          R om = R(1) - s;
-          R r = Ar<R>::div(s, om);
-          dq = Ar<R>::div(qv - r * gsum, R(1) + Ar<R>::div(s, om * om) * bt * alpha * gsum);
-        }
-        R drho;
-        if (dq >= qv) {
-          dq = qv;
-          drho = y[1 + i];
-        } else if (dq <= -qc) {
-          dq = -qc;
-          drho = -y[L::cond(i, 0)];
-        } else {
-          drho = dq * C.eps[i] * N;
-        }
-        if (drho != R(0)) {
-          const R yv = y[1 + i], yc = y[L::cond(i, 0)];
-          y[1 + i] -= drho;
-          y[L::cond(i, 0)] += drho;
-          // the changes as stored (after rounding to the state's type)
-          if constexpr (sizeof(R) == 4) {
-            // FP32 states: the increments in FP32 (good to ~1e-7 of themselves, ~1e-10 of T),
-            // accumulated into the FP64 T, heat capacity and gas sum
-            const R dv = y[1 + i] - yv, dc = y[L::cond(i, 0)] - yc;
-            const R dC = (C.sig_v[i] * dv + C.sig_c[i][0] * dc) * C.c_vd;
-            const R dT = (C.mu[i][0] * dc + R(Td) * dC) * Ar<R>::rcp(R(Cvd) + dC);
-            Td -= double(dT);
-            Cvd += double(dC);
-            Rmd += double(C.inv_eps[i] * dv);
-          } else {
-            const double dv = double(y[1 + i]) - double(yv);
-            const double dc = double(y[L::cond(i, 0)]) - double(yc);
-            const double dC = (ph.sig_v[i] * dv + ph.sig_c[i][0] * dc) * ph.c_vd;
-            Td -= quot64<R>(ph.mu[i][0] * dc + Td * dC, Cvd + dC);
-            Cvd += dC;
-            Rmd += ph.inv_eps[i] * dv;
-          }
-          pd = Rmd * ph.R_d * Td;
-        }
-        if (fabs(dq) > tol * (qv + qc)) conv = false;
-      }
-      if (conv) return sweep;
-    }
-    return -1;
+    return satadj_sweeps<R, L>(ph, C, y, eref, max_iter);
   }
 }
 
@@ -743,29 +821,31 @@ __device__ __forceinline__ void sediment_flux(const CstT<R> &C, const R *XL, con
 // Jacobian (rho* varies with T, which the reactions change at fixed rho e: dT/drho_k =
 // -(mu_k + c_k T)/C_v), one form of the rates at a time: the form of the initial state, then
 // the other if the result lies on the wrong side of saturation, else the saturated form.
-// T is inverted from the energy in FP64. Returns the largest iteration count or -1.
+// T is inverted from the energy in wide numbers. Returns the largest iteration count or -1.
 // ------------------------------------------------------------------------------------------
 template <class R, class L>
 __device__ __forceinline__ void kessler_eval(const Phys &ph, const CstT<R> &C, const R *y,
-                                             double T0, R Cv0, int i, R rho, const R *yn, R dt,
+                                             typename Wide<R>::T T0w, R Cv0, int i, R rho,
+                                             const R *yn, R dt,
                                              bool sat, R G[2], R A[2][2], R &s_out,
                                              R &tol_out) {
   const int vi = 1 + i, ci = L::cond(i, 0), ri = L::cond(i, 1);
-  // T from T0, the FP64 temperature of the densities yn this vapour started from, and the
+  // T from T0, the wide temperature of the densities yn this vapour started from, and the
   // phase changes since: rho e and the momenta are fixed, so C_v T + A is (Sec. 2), and
   // T = T0 - (sum_k mu_k d_k + T0 sum_k c_k d_k) / (C_v0 + sum_k c_k d_k) over the vapour,
-  // cloud and precipitation changes d_k (the vapour's mu is zero) -- no FP64 inversion per
+  // cloud and precipitation changes d_k (the vapour's mu is zero) -- no inversion per
   // Newton iteration
+  const R T0 = Wide<R>::r(T0w);
   const R dv = y[vi] - yn[0], dc = y[ci] - yn[1], dr = y[ri] - yn[2];
   const R dC = (C.sig_v[i] * dv + C.sig_c[i][0] * dc + C.sig_c[i][1] * dr) * C.c_vd;
   const R dA = C.mu[i][0] * dc + C.mu[i][1] * dr;
-  const R incr = -(dA + R(T0) * dC) * Ar<R>::rcp(Cv0 + dC);
-  const R T = R(T0) + incr, iT = Ar<R>::rcp(T), t = T * C.inv_Tref[i], it = Ar<R>::rcp(t);
-  // T - T^r kept accurate (T0 - T^r from the FP64 temperature): rho*(T) is steep,
+  const R incr = -(dA + T0 * dC) * Ar<R>::rcp(Cv0 + dC);
+  const R T = T0 + incr, iT = Ar<R>::rcp(T), t = T * C.inv_Tref[i], it = Ar<R>::rcp(t);
+  // T - T^r kept accurate (T0 - T^r from the wide temperature): rho*(T) is steep,
   // d ln rho*/d ln T ~ beta / t ~ 20 near water's triple point, so T rounded to FP32 alone
   // would put ~1e-6 relative noise into s = rho_v - rho* -- the size of the FP32 Newton stop
   // tolerance
-  const R dTr = R(T0 - ph.Tref[i]) + incr;
+  const R dTr = Wide<R>::r(T0w - Wide<R>::Tref(ph, C, i)) + incr;
   const R arg = C.beta[i] * dTr * iT - C.delta[i] * Ar<R>::log1p_(dTr * C.inv_Tref[i]);
   const R rs = C.pref[i] * Ar<R>::exp_(arg) * C.eps[i] * C.iR_d * iT;  // p* / (R_i T)
   // rho* is held only to ~(|arg| + 2) eps relative: the Newton stop test allows 4 times it
@@ -820,7 +900,8 @@ __device__ __forceinline__ void kessler_eval(const Phys &ph, const CstT<R> &C, c
 
 template <class R, class L>
 __device__ __forceinline__ int kessler_branch(const Phys &ph, const CstT<R> &C, R *y,
-                                              double T0, R Cv0, int i, R rho, const R *yn,
+                                              typename Wide<R>::T T0, R Cv0, int i, R rho,
+                                              const R *yn,
                                               R tot, R dt, bool sat, R &s) {
   const int vi = 1 + i, ci = L::cond(i, 0), ri = L::cond(i, 1);
   y[vi] = yn[0];
@@ -845,24 +926,26 @@ __device__ __forceinline__ int kessler_branch(const Phys &ph, const CstT<R> &C, 
 }
 
 template <class R, class L>
-__device__ int kessler_cell(const Phys &ph, const CstT<R> &C, R *y, double eref, R dt) {
+__device__ int kessler_cell(const Phys &ph, const CstT<R> &C, R *y, typename Wide<R>::T eref,
+                            R dt) {
   if constexpr (!(L::NVAP > 0 && L::NCOND >= 2)) {
     return 0;
   } else {
     R rho = R(0);
 #pragma unroll
     for (int s = 0; s < L::IM0; ++s) rho += y[s];
-    // the cell's temperature and heat capacity once in FP64; each vapour then updates them
-    // by its own phase changes
-    double T0, p0, Cv0;
-    cell_Tp<R, L>(ph, y, eref, T0, p0, &Cv0);
+    // the cell's temperature and heat capacity once in wide numbers; each vapour then updates
+    // them by its own phase changes
+    using W = Wide<R>;
+    typename W::T T0, Cv0, Rm0;
+    invert_T<R, L>(ph, C, y, eref, T0, Cv0, Rm0);
     int worst = 0;
     for (int i = 0; i < L::NVAP; ++i) {
       const int vi = 1 + i, ci = L::cond(i, 0), ri = L::cond(i, 1);
       const R yn[3] = {y[vi], y[ci], y[ri]};
       const R tot = yn[0] + yn[1] + yn[2];
       R G[2], A[2][2], s0, s, tol0;
-      const R cv0 = R(Cv0);
+      const R cv0 = W::r(Cv0);
       kessler_eval<R, L>(ph, C, y, T0, cv0, i, rho, yn, dt, true, G, A, s0, tol0);
       const bool first = s0 > R(0);
       int it = kessler_branch<R, L>(ph, C, y, T0, cv0, i, rho, yn, tot, dt, first, s);
@@ -871,13 +954,14 @@ __device__ int kessler_cell(const Phys &ph, const CstT<R> &C, R *y, double eref,
         if (!(it > 0 && (!first ? s > R(0) : s <= R(0))))
           it = kessler_branch<R, L>(ph, C, y, T0, cv0, i, rho, yn, tot, dt, true, s);
       }
-      {  // this vapour's phase changes, in FP64, carried to the next vapour's T0 and C_v0
-        const double dv = double(y[vi]) - double(yn[0]), dc = double(y[ci]) - double(yn[1]);
-        const double dr = double(y[ri]) - double(yn[2]);
-        const double dC = (ph.sig_v[i] * dv + ph.sig_c[i][0] * dc + ph.sig_c[i][1] * dr) * ph.c_vd;
-        const double dA = ph.mu[i][0] * dc + ph.mu[i][1] * dr;
-        T0 -= quot64<R>(dA + T0 * dC, Cv0 + dC);
-        Cv0 += dC;
+      {  // this vapour's phase changes, in wide numbers, carried to the next vapour's T0 and C_v0
+        const typename W::T dv = W::diff(y[vi], yn[0]), dc = W::diff(y[ci], yn[1]);
+        const typename W::T dr = W::diff(y[ri], yn[2]);
+        const typename W::T dC = (W::sig_v(ph, C, i) * dv + W::sig_c(ph, C, i, 0) * dc +
+                                  W::sig_c(ph, C, i, 1) * dr) * W::c_vd(ph, C);
+        const typename W::T dA = W::mu(ph, C, i, 0) * dc + W::mu(ph, C, i, 1) * dr;
+        T0 = T0 - W::quot(dA + T0 * dC, Cv0 + dC);
+        Cv0 = Cv0 + dC;
       }
       if (it < 0)
         worst = -1;
@@ -1149,6 +1233,193 @@ __device__ __forceinline__ void grid_barrier(GridSync *gs, unsigned int nblocks,
   __syncthreads();
 }
 
+// The stage's time step (one thread per CTA). The first tile of a domain records it in stage 0 and
+// clears the domain's CFL maximum in stage 1; kept is the CTA's own stage-0 time step (resident
+// step, stages 1 and 2).
+template <bool RES>
+__device__ __forceinline__ double stage_dt(const StageArgs &a, const DomDev &D, int stage, int lt,
+                                           double kept) {
+  if (stage == 0) {
+    const double dt = a.dt_override > 0.0 ? a.dt_override
+                      : (D.dt_fixed > 0.0 ? D.dt_fixed
+                                          : D.cfl / __longlong_as_double((long long)*D.rate));
+    if (lt == 0) *D.dt_step = dt;
+    return dt;
+  }
+  if (RES) return kept;
+  if (stage == 1 && lt == 0) *D.rate = 0ull;
+  return *(volatile double *)D.dt_step;
+}
+
+// Where the cell (gx, gy, gz) beyond a tile along direction dirn (it may lie outside the domain, at
+// most 3 cells) takes its values from: the interior cell itself, a slab neighbour's cell, or for
+// a ghost of the domain boundary the cell it wraps to or mirrors (flip). Field v is src[v * stride].
+template <class R>
+struct HaloCell {
+  const R *src;
+  long long stride;
+  int side;  // the domain side along dirn that a ghost lies beyond (x-, x+, y-, y+, z-, z+)
+  int gz;    // level of the source cell
+  bool flip;
+};
+template <class R>
+__device__ __forceinline__ HaloCell<R> halo_cell(const StageArgs &a, const DomDev &D, int stage,
+                                                 const R *Ys, int gx, int gy, int gz, int dirn) {
+  HaloCell<R> h;
+  const int nx = D.nx, ny = D.ny, nz = D.nz;
+  h.side = 2 * dirn + ((dirn == 0 ? gx : (dirn == 1 ? gy : gz)) < 0 ? 0 : 1);
+  h.flip = false;
+  if (dirn == 0 && (gx < 0 || gx >= nx) && D.bc[h.side] == kBcHalo && !a.buf_s) {
+    // a slab boundary: the neighbouring slab's cells (a linked domain's stage input, or the
+    // ghost buffer the caller filled)
+    const int s = h.side, hn = D.hnx[s];
+    h.stride = (long long)hn * ny * nz;
+    h.src = reinterpret_cast<const R *>(D.hsrc[s][stage]) + ((long long)gz * ny + gy) * hn +
+            D.hoff[s] + (s ? gx - nx : gx + 3);
+  } else {
+    if (dirn == 0) gx = map_index(gx, nx, D.bc[0], D.bc[1], h.flip);
+    if (dirn == 1) gy = map_index(gy, ny, D.bc[2], D.bc[3], h.flip);
+    if (dirn == 2) gz = map_index(gz, nz, D.bc[4], D.bc[5], h.flip);
+    h.stride = D.ncell;
+    h.src = Ys + (((long long)gz * ny + gy) * nx + gx);
+  }
+  h.gz = gz;
+  return h;
+}
+// Its conserved values; CG reads past L1 (cells other CTAs wrote during this launch).
+template <class R, int NV, bool CG>
+__device__ __forceinline__ void load_fields(const R *src, long long stride, R *y) {
+#pragma unroll
+  for (int v = 0; v < NV; ++v) y[v] = CG ? __ldcg(src + v * stride) : src[v * stride];
+}
+// Its primitives from those values: a wall's ghost has the normal velocity, or at a no-slip wall
+// every component, negated, and below a fixed-temperature floor the temperature T_bot.
+template <class R, class L, class DD>
+__device__ __forceinline__ void halo_prim(const DD &D, const Phys &ph, const CstT<R> &C,
+                                          const HaloCell<R> &h, int dirn, const R *y, R *x, R &pt) {
+  R Tt;
+  cons_to_prim<R, L>(ph, C, D, h.gz, y, x, pt, Tt);
+  if (h.flip) {
+    // (selects, not x[mom(dirn)]: a run-time index would put x into local memory)
+    const bool all = D.bc[h.side] == kBcNoSlip;
+#pragma unroll
+    for (int m = L::IM0; m < L::IM0 + L::NMOM; ++m)
+      if (all || m == L::mom(dirn)) x[m] = -x[m];
+    // Sec. 6 lower boundary: the ghost holds T_bot at the mirrored pressure and composition,
+    // so its density is p / (R_d den T_bot) (App. B: p = rho R_d den T, den the mixing
+    // factor), the mirrored density times T / T_bot
+    if (h.side == 4 && D.T_bot > 0.0) {
+      R num, den;
+      mix_factors<R, L>(C, x, num, den);
+      x[0] = pt * C.iR_d * Ar<R>::rcp(den * R(D.T_bot));
+    }
+  }
+}
+
+// Both face states of the cell whose five-cell window is at locations o of the grouped array
+// base (N locations): one group of fields at a time (the group's five window points, one vector
+// access each); FP32 pairs on the packed FP32x2 pipe, an odd field alone.
+template <class R, int NV>
+__device__ __forceinline__ void recon_window(const R *base, const int (&o)[5], int N, R weps,
+                                             R *QM, R *QP) {
+  using V = SV<R, NV>;
+#pragma unroll
+  for (int g = 0; g < V::NF + V::T2 + V::T1; ++g) {
+    const int f0 = g < V::NF ? g * V::W : (g == V::NF && V::T2 ? V::P2 : V::P1);
+    const int n = g < V::NF ? V::W : (g == V::NF && V::T2 ? 2 : 1);
+    R X[5][V::W];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) V::load_group(base, g, o[k], N, X[k]);
+    if constexpr (sizeof(R) == 4) {
+#pragma unroll
+      for (int j = 0; j + 1 < V::W; j += 2) {
+        if (j + 1 < n) {
+          float2 qm, qp;
+          weno5_pair2(make_float2(X[0][j], X[0][j + 1]), make_float2(X[1][j], X[1][j + 1]),
+                      make_float2(X[2][j], X[2][j + 1]), make_float2(X[3][j], X[3][j + 1]),
+                      make_float2(X[4][j], X[4][j + 1]), weps, qm, qp);
+          QM[f0 + j] = qm.x, QM[f0 + j + 1] = qm.y, QP[f0 + j] = qp.x, QP[f0 + j + 1] = qp.y;
+        }
+      }
+      if (n == 1)
+        weno5_pair<R>(X[0][0], X[1][0], X[2][0], X[3][0], X[4][0], weps, QM[f0], QP[f0]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < V::W; ++j)
+        if (j < n)
+          weno5_pair<R>(X[0][j], X[1][j], X[2][j], X[3][j], X[4][j], weps, QM[f0 + j], QP[f0 + j]);
+    }
+  }
+}
+
+// The end of a cell's stage: gravity and forcing added to the flux divergence acc, the stage
+// combine, saturation adjustment, microphysics (stage 2) and the checks of the result yo. ys is
+// the stage input, yn(v) field v of Y^n (stages 1 and 2), mb and mt the total-mass fluxes
+// through the cell's lower and upper z faces.
+template <class R, class L, bool MICRO, class DD, class YN>
+__device__ __forceinline__ void finish_cell(const StageArgs &a, const DD &D, const Phys &ph,
+                                            const CstT<R> &C, int stage, R dt, int k, const R *ys,
+                                            R *acc, R mb, R mt, YN yn, R *yo) {
+  using P = Prof<R>;
+  const R grav = P::grav(D);
+  // vertical momentum: -(rho - rho_bar) g (Eq. mom3 with the reference balance removed)
+  acc[L::mom(2)] -= P::template drho<L>(D, k, ys) * grav;
+  // energy: -g (F_rho,k-1/2 + F_rho,k+1/2) / 2 with the vertical total-mass fluxes
+  acc[L::IE] -= grav * R(0.5) * (mb + mt);
+  if constexpr (MICRO && L::MOIST) {
+    // forcing of the Jovian simulation (Sec. 6) by the level's reference pressure
+    const R pk = P::pc(D, k);
+    if (C.cool_rate != R(0) && pk >= C.cool_p_lo && pk <= C.cool_p_hi) {
+      R Cv = ys[0];  // heat capacity at constant volume / c_vd
+#pragma unroll
+      for (int i2 = 0; i2 < L::NVAP; ++i2) {
+        Cv += C.sig_v[i2] * ys[1 + i2];
+#pragma unroll
+        for (int j2 = 0; j2 < L::NCOND; ++j2) Cv += C.sig_c[i2][j2] * ys[L::cond(i2, j2)];
+      }
+      acc[L::IE] -= Cv * C.c_vd * C.cool_rate;
+    }
+    if (C.sponge_itau0 != R(0) && pk * C.sponge_ip0 < R(1)) {
+      const R r = pk * C.sponge_ip0, rate = C.sponge_itau0 * Ar<R>::rcp(r * r);
+      acc[L::mom(0)] -= ys[L::mom(0)] * rate;
+      if constexpr (L::D3) acc[L::mom(1)] -= ys[L::mom(1)] * rate;
+    }
+  }
+#pragma unroll
+  for (int v = 0; v < L::NV; ++v) {
+    const R s1 = ys[v] + dt * acc[v];
+    if (stage == 0) {
+      yo[v] = s1;
+    } else {
+      // (1 - w) Y^n + w s1 as Y^n + w (s1 - Y^n): the two weights sum to exactly one. With 1/3
+      // and 2/3 each rounded to FP32 they sum to 1 + 3e-8, which scales the whole state by that
+      // much every step (a mass drift of 1e-3 over 30,000 steps). An explicit fused
+      // multiply-add, so that every kernel that inlines this rounds it the same way.
+      const R y0 = yn(v), wgt = stage == 1 ? R(0.25) : R(2.0 / 3.0);
+      yo[v] = fma(wgt, s1 - y0, y0);
+    }
+  }
+  if constexpr (L::MOIST) {
+    if (ph.satadj) {
+      const int it = satadj_cell<R, L>(ph, C, yo, Wide<R>::e_ref(D, k), P::er(D, k),
+                                          ph.satadj_max_iter);
+      if (it < 0)
+        atomicOr(a.flags, (unsigned)kFlagNoConv);
+      else if (it > 2)
+        atomicMax(a.max_sweeps, it);
+    }
+    // the microphysics follows each step (time splitting), over the step's dt
+    if (MICRO && stage == 2 && ph.kessler) {
+      if (kessler_cell<R, L>(ph, C, yo, Wide<R>::e_ref(D, k), dt) < 0)
+        atomicOr(a.flags, (unsigned)kFlagNoConv);
+    }
+  }
+  R rs = R(0);
+#pragma unroll
+  for (int s = 0; s < L::IM0; ++s) rs += yo[s];
+  if (!(rs > R(0)) || !isfinite(yo[L::IE])) atomicOr(a.flags, (unsigned)kFlagNonFinite);
+}
+
 // One stage over the CTA's tiles. RES (the resident step, one tile per CTA for all three
 // stages): for stages 1 and 2 ys holds the owned cells' stage input on entry (the previous
 // stage's output, kept in registers) instead of being loaded; Y^n of the owned cells is kept
@@ -1192,20 +1463,7 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
     const R *Yn = reinterpret_cast<const R *>(a.buf_n ? a.buf_n : D.buf[0]);
     R *Yo = reinterpret_cast<R *>(a.buf_o ? a.buf_o : D.buf[stage == 0 ? 1 : (stage == 1 ? 2 : 0)]);
     // the stage's time step, formed once per CTA
-    if (tid == 0) {
-      double dt;
-      if (stage == 0) {
-        dt = a.dt_override > 0.0 ? a.dt_override
-             : (D.dt_fixed > 0.0 ? D.dt_fixed : D.cfl / __longlong_as_double((long long)*D.rate));
-        if (lt == 0) *D.dt_step = dt;
-      } else if (!RES) {
-        dt = *(volatile double *)D.dt_step;
-        if (stage == 1 && lt == 0) *D.rate = 0ull;
-      } else {
-        dt = s_red[0];  // this CTA's own stage-0 time step
-      }
-      s_red[0] = dt;
-    }
+    if (tid == 0) s_red[0] = stage_dt<RES>(a, D, stage, lt, s_red[0]);
 
     // ---- 1. owned cells: load, keep the conserved values, store primitives -------------
     if constexpr (S::PREFETCH && !RES) {
@@ -1281,51 +1539,11 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
           dirn = 2;
         }
         if (!ok) continue;
-        int gx = x0 + bx - 3, gy = y0 + by - B::HY, gz = z0 + bz - 3;
-        // the side this ghost lies beyond (x-, x+, y-, y+, z-, z+)
-        const int side = 2 * dirn + ((dirn == 0 ? gx : (dirn == 1 ? gy : gz)) < 0 ? 0 : 1);
-        bool flip = false;
-        const R *src = Ys;
-        long long g, nsrc = ncell;
-        if (dirn == 0 && (gx < 0 || gx >= nx) && D.bc[side] == kBcHalo && !a.buf_s) {
-          // a slab boundary: the neighbouring slab's cells (a linked domain's stage input,
-          // or the ghost buffer the caller filled)
-          const int h = side, hn = D.hnx[h];
-          src = reinterpret_cast<const R *>(D.hsrc[h][stage]);
-          nsrc = (long long)hn * ny * nz;
-          g = ((long long)gz * ny + gy) * hn + D.hoff[h] + (h ? gx - nx : gx + 3);
-        } else {
-          if (dirn == 0) gx = map_index(gx, nx, D.bc[0], D.bc[1], flip);
-          if (dirn == 1) gy = map_index(gy, ny, D.bc[2], D.bc[3], flip);
-          if (dirn == 2) gz = map_index(gz, nz, D.bc[4], D.bc[5], flip);
-          g = ((long long)gz * ny + gy) * nx + gx;
-        }
-        R y[NV], x[NV], pt, Tt;
-        if constexpr (RES) {
-#pragma unroll
-          for (int v = 0; v < NV; ++v) y[v] = __ldcg(src + v * nsrc + g);
-        } else {
-#pragma unroll
-          for (int v = 0; v < NV; ++v) y[v] = src[v * nsrc + g];
-        }
-        cons_to_prim<R, L>(ph, C, D, gz, y, x, pt, Tt);
-        if (flip) {
-          // a wall: free-slip negates the normal velocity, no-slip every component
-          if (D.bc[side] == kBcNoSlip) {
-#pragma unroll
-            for (int m = 0; m < L::NMOM; ++m) x[L::IM0 + m] = -x[L::IM0 + m];
-          } else {
-            x[L::mom(dirn)] = -x[L::mom(dirn)];
-          }
-          // Sec. 6 lower boundary: the ghost holds T_bot at the mirrored pressure and
-          // composition, so its density is p / (R_d den T_bot) (App. B: p = rho R_d den T,
-          // den the mixing factor), the mirrored density times T / T_bot
-          if (side == 4 && D.T_bot > 0.0) {
-            R num, den;
-            mix_factors<R, L>(C, x, num, den);
-            x[0] = pt * C.iR_d * Ar<R>::rcp(den * R(D.T_bot));
-          }
-        }
+        const HaloCell<R> hc =
+            halo_cell<R>(a, D, stage, Ys, x0 + bx - 3, y0 + by - B::HY, z0 + bz - 3, dirn);
+        R y[NV], x[NV], pt;
+        load_fields<R, NV, RES>(hc.src, hc.stride, y);
+        halo_prim<R, L>(D, ph, C, hc, dirn, y, x, pt);
         const int bi = B::idx(bx, by, bz);
         V::store(s_prim, bi, B::NSTORE, x);
         // the viscous heat flux reads theta and the Exner function only on the two sides of
@@ -1389,36 +1607,7 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
             const int fr = (lz * sy + ly) * sx + lx;                        // face c-1/2
             const bool has_l = ld < ed, has_r = ld >= 0;
             R QM[NV], QP[NV];
-            // one group of fields at a time (the group's five window points, one vector access
-            // each): FP32 pairs on the packed FP32x2 pipe, an odd field alone
-#pragma unroll
-            for (int g = 0; g < V::NF + V::T2 + V::T1; ++g) {
-              const int f0 = g < V::NF ? g * V::W : (g == V::NF && V::T2 ? V::P2 : V::P1);
-              const int n = g < V::NF ? V::W : (g == V::NF && V::T2 ? 2 : 1);
-              R X[5][V::W];
-#pragma unroll
-              for (int k = 0; k < 5; ++k) V::load_group(s_prim, g, o[k], B::NSTORE, X[k]);
-              if constexpr (sizeof(R) == 4) {
-#pragma unroll
-                for (int j = 0; j + 1 < V::W; j += 2) {
-                  if (j + 1 < n) {
-                    float2 qm, qp;
-                    weno5_pair2(make_float2(X[0][j], X[0][j + 1]), make_float2(X[1][j], X[1][j + 1]),
-                                make_float2(X[2][j], X[2][j + 1]), make_float2(X[3][j], X[3][j + 1]),
-                                make_float2(X[4][j], X[4][j + 1]), weps, qm, qp);
-                    QM[f0 + j] = qm.x, QM[f0 + j + 1] = qm.y, QP[f0 + j] = qp.x, QP[f0 + j + 1] = qp.y;
-                  }
-                }
-                if (n == 1)
-                  weno5_pair<R>(X[0][0], X[1][0], X[2][0], X[3][0], X[4][0], weps, QM[f0], QP[f0]);
-              } else {
-#pragma unroll
-                for (int j = 0; j < V::W; ++j)
-                  if (j < n)
-                    weno5_pair<R>(X[0][j], X[1][j], X[2][j], X[3][j], X[4][j], weps, QM[f0 + j],
-                                  QP[f0 + j]);
-              }
-            }
+            recon_window<R, NV>(s_prim, o, B::NSTORE, weps, QM, QP);
             if (has_l) V::store(s_fl, fl, B::NF, QM);
             if (has_r) V::store(s_fr, fr, B::NF, QP);
           }
@@ -1499,10 +1688,7 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
       const int lx = c % TX, ly = (c / TX) % TY, lz = c / (TX * TY);
       if (c < B::NCELL && lx < ex && ly < ey && lz < ez) {
         const int k = z0 + lz;
-        const R grav = P::grav(D);
-        // vertical momentum: -(rho - rho_bar) g (Eq. mom3 with the reference balance removed)
-        acc[m][L::mom(2)] -= P::template drho<L>(D, k, ys[m]) * grav;
-        // energy: -g (F_rho,k-1/2 + F_rho,k+1/2) / 2 with the vertical total-mass fluxes
+        // vertical total-mass fluxes through the cell's two z faces
         const int f0 = (lz * TY + ly) * TX + lx;
         const int f1 = ((lz + 1) * TY + ly) * TX + lx;
         R mb = R(0), mt = R(0);
@@ -1511,63 +1697,11 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
           mb += s_fl[V::at(s, f0, B::NF)];
           mt += s_fl[V::at(s, f1, B::NF)];
         }
-        acc[m][L::IE] -= grav * R(0.5) * (mb + mt);
-        if constexpr (MICRO && L::MOIST) {
-          // forcing of the Jovian simulation (Sec. 6) by the level's reference pressure
-          const R pk = P::pc(D, k);
-          if (C.cool_rate != R(0) && pk >= C.cool_p_lo && pk <= C.cool_p_hi) {
-            R Cv = ys[m][0];  // heat capacity at constant volume / c_vd
-#pragma unroll
-            for (int i2 = 0; i2 < L::NVAP; ++i2) {
-              Cv += C.sig_v[i2] * ys[m][1 + i2];
-#pragma unroll
-              for (int j2 = 0; j2 < L::NCOND; ++j2) Cv += C.sig_c[i2][j2] * ys[m][L::cond(i2, j2)];
-            }
-            acc[m][L::IE] -= Cv * C.c_vd * C.cool_rate;
-          }
-          if (C.sponge_itau0 != R(0) && pk * C.sponge_ip0 < R(1)) {
-            const R r = pk * C.sponge_ip0, rate = C.sponge_itau0 * Ar<R>::rcp(r * r);
-            acc[m][L::mom(0)] -= ys[m][L::mom(0)] * rate;
-            if constexpr (L::D3) acc[m][L::mom(1)] -= ys[m][L::mom(1)] * rate;
-          }
-        }
         const long long g = ((long long)k * ny + (y0 + ly)) * nx + (x0 + lx);
         R yo[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-          const R s1 = ys[m][v] + dt * acc[m][v];
-          if (stage == 0) {
-            yo[v] = s1;
-          } else {
-            const R yn = S::PREFETCH ? s_yn[v * B::NCELL + c] : Yn[v * ncell + g];
-            // (1 - w) Y^n + w s1 as Y^n + w (s1 - Y^n): the two weights sum to exactly one.
-            // With 1/3 and 2/3 each rounded to FP32 they sum to 1 + 3e-8, which scales the
-            // whole state by that much every step (a mass drift of 1e-3 over 30,000 steps)
-            // (an explicit fused multiply-add, so that every kernel that inlines this rounds
-            // it the same way)
-            const R wgt = stage == 1 ? R(0.25) : R(2.0 / 3.0);
-            yo[v] = fma(wgt, s1 - yn, yn);
-          }
-        }
-        if constexpr (L::MOIST) {
-          if (ph.satadj) {
-            const int it =
-                satadj_cell<R, L>(ph, C, yo, D.e_ref[k], P::er(D, k), ph.satadj_max_iter);
-            if (it < 0)
-              atomicOr(a.flags, (unsigned)kFlagNoConv);
-            else if (it > 2)
-              atomicMax(a.max_sweeps, it);
-          }
-          // the microphysics follows each step (time splitting), over the step's dt
-          if (MICRO && stage == 2 && ph.kessler) {
-            if (kessler_cell<R, L>(ph, C, yo, D.e_ref[k], dt) < 0)
-              atomicOr(a.flags, (unsigned)kFlagNoConv);
-          }
-        }
-        R rs = R(0);
-#pragma unroll
-        for (int s = 0; s < L::IM0; ++s) rs += yo[s];
-        if (!(rs > R(0)) || !isfinite(yo[L::IE])) atomicOr(a.flags, (unsigned)kFlagNonFinite);
+        finish_cell<R, L, MICRO>(
+            a, D, ph, C, stage, dt, k, ys[m], acc[m], mb, mt,
+            [&](int v) { return S::PREFETCH ? s_yn[v * B::NCELL + c] : Yn[v * ncell + g]; }, yo);
 #pragma unroll
         for (int v = 0; v < NV; ++v) Yo[v * ncell + g] = yo[v];
         if constexpr (RES) {
@@ -1592,12 +1726,38 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
   }
 }
 
+// The march along z (snap_march.cuh), for the tile shapes that ask for it.
+template <class R, class L, class T>
+struct MarchSmem;
+template <class R, class L, class T, bool MICRO, bool RES>
+__device__ __forceinline__ void march_tiles(const StageArgs &a, const int stage,
+                                            unsigned char *smem);
+
+// One stage over the CTA's tiles by the tile shape's method; st 0, 1, 2.
+template <class R, class L, bool VISC, class T, bool MICRO>
+__device__ __forceinline__ void run_stage(const StageArgs &a, int st, unsigned char *smem) {
+  if constexpr (T::MARCH) {
+    static_assert(!VISC, "the march is built for inviscid layouts");
+    march_tiles<R, L, T, MICRO, false>(a, st, smem);
+  } else {
+    R ys[Box<T, L::D3>::CPT][L::NV];
+    stage_tiles<R, L, VISC, T, MICRO>(a, st, smem, ys);
+  }
+}
+
+template <class R, class L, bool VISC, class T>
+constexpr size_t stage_smem() {
+  if constexpr (T::MARCH)
+    return MarchSmem<R, L, T>::total;
+  else
+    return StageSmem<R, L, VISC, T>::total;
+}
+
 // One Runge-Kutta stage over all tiles of all domains.
 template <class R, class L, bool VISC, class T, bool MICRO>
 __global__ void __launch_bounds__(T::NT, T::MINB) stage_kernel(const StageArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  R ys[Box<T, L::D3>::CPT][L::NV];
-  stage_tiles<R, L, VISC, T, MICRO>(a, a.stage, smem, ys);
+  run_stage<R, L, VISC, T, MICRO>(a, a.stage, smem);
 }
 
 // One whole step (three stages) in a single persistent cooperative launch: the CTAs walk the
@@ -1605,10 +1765,9 @@ __global__ void __launch_bounds__(T::NT, T::MINB) stage_kernel(const StageArgs a
 template <class R, class L, bool VISC, class T, bool MICRO>
 __global__ void __launch_bounds__(T::NT, T::MINB) step_kernel(const StageArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
-  R ys[Box<T, L::D3>::CPT][L::NV];
 #pragma unroll 1
   for (int st = 0; st < 3; ++st) {
-    stage_tiles<R, L, VISC, T, MICRO>(a, st, smem, ys);
+    run_stage<R, L, VISC, T, MICRO>(a, st, smem);
     if (st < 2) grid_barrier(a.gsync, gridDim.x, a.flags, a.spin_limit, a.absent_cta);
   }
 }
@@ -1623,7 +1782,7 @@ template <class R, class L, bool VISC, class T, bool MICRO>
 __global__ void __launch_bounds__(T::NT, T::MINB) resident_step_kernel(const StageArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned int s_seq;
-  R ys[Box<T, L::D3>::CPT][L::NV];
+  R ys[T::MARCH ? 1 : Box<T, L::D3>::CPT][L::NV];
   const int tile = blockIdx.x, tid = threadIdx.x;
   if (tid == 0) s_seq = ld_acquire_u32(&a.res->seq);
   __syncthreads();
@@ -1647,7 +1806,11 @@ __global__ void __launch_bounds__(T::NT, T::MINB) resident_step_kernel(const Sta
       }
       __syncthreads();
     }
-    stage_tiles<R, L, VISC, T, MICRO, true>(a, st, smem, ys);  // ends with a CTA barrier
+    // either ends with a CTA barrier
+    if constexpr (T::MARCH)
+      march_tiles<R, L, T, MICRO, true>(a, st, smem);
+    else
+      stage_tiles<R, L, VISC, T, MICRO, true>(a, st, smem, ys);
     if (st < 2 && tid == 0) {
       __threadfence();
       st_release_u32(a.tile_flags + tile, 3u * seq + unsigned(st) + 1u);
@@ -1805,9 +1968,8 @@ __global__ void __launch_bounds__(256) satadj_kernel(const StageArgs a, int dm, 
     R y[L::NV];
 #pragma unroll
     for (int v = 0; v < L::NV; ++v) y[v] = Y[v * D.ncell + c];
-    const double er = D.e_ref[c / ((long long)D.nx * D.ny)];
-    const int it = satadj_cell<R, L>(a.ph, cst<R>(a), y, er,
-                                     Prof<R>::er(D, int(c / ((long long)D.nx * D.ny))),
+    const int k = int(c / ((long long)D.nx * D.ny));
+    const int it = satadj_cell<R, L>(a.ph, cst<R>(a), y, Wide<R>::e_ref(D, k), Prof<R>::er(D, k),
                                      a.ph.satadj_max_iter);
     if (it < 0)
       atomicOr(a.flags, (unsigned)kFlagNoConv);
@@ -1823,17 +1985,17 @@ __global__ void __launch_bounds__(256) satadj_kernel(const StageArgs a, int dm, 
 // ------------------------------------------------------------------------------------------
 template <class R, class L, bool VISC, class T, bool MICRO = false>
 struct Variant {
-  using S = StageSmem<R, L, VISC, T>;
+  static constexpr size_t kSmem = stage_smem<R, L, VISC, T>();
   static cudaError_t prepare() {
     cudaError_t e = cudaFuncSetAttribute(stage_kernel<R, L, VISC, T, MICRO>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         int(S::total));
+                                         int(kSmem));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(resident_step_kernel<R, L, VISC, T, MICRO>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::total));
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(step_kernel<R, L, VISC, T, MICRO>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::total));
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
   }
   static int max_resident_tiles() {
     int dev = 0, nsm = 0, per = 0;
@@ -1841,7 +2003,7 @@ struct Variant {
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per, resident_step_kernel<R, L, VISC, T, MICRO>, T::NT, S::total) != cudaSuccess)
+            &per, resident_step_kernel<R, L, VISC, T, MICRO>, T::NT, kSmem) != cudaSuccess)
       return 0;
     return per * nsm;
   }
@@ -1849,7 +2011,7 @@ struct Variant {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(T::NT);
-    cfg.dynamicSmemBytes = S::total;
+    cfg.dynamicSmemBytes = kSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -1859,7 +2021,7 @@ struct Variant {
     return cudaLaunchKernelEx(&cfg, resident_step_kernel<R, L, VISC, T, MICRO>, a);
   }
   static cudaError_t stage(const StageArgs &a, int grid, cudaStream_t s) {
-    stage_kernel<R, L, VISC, T, MICRO><<<grid, T::NT, S::total, s>>>(a);
+    stage_kernel<R, L, VISC, T, MICRO><<<grid, T::NT, kSmem, s>>>(a);
     return cudaGetLastError();
   }
   static int max_resident_blocks() {
@@ -1868,7 +2030,7 @@ struct Variant {
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, step_kernel<R, L, VISC, T, MICRO>, T::NT,
-                                                      S::total) != cudaSuccess)
+                                                      kSmem) != cudaSuccess)
       return 0;
     return per * nsm;
   }
@@ -1876,7 +2038,7 @@ struct Variant {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(T::NT);
-    cfg.dynamicSmemBytes = S::total;
+    cfg.dynamicSmemBytes = kSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
@@ -1890,8 +2052,9 @@ struct Variant {
     v.tile[0] = T::TX;
     v.tile[1] = T::TY;
     v.tile[2] = T::TZ;
+    v.march = T::MARCH;
     v.threads = T::NT;
-    v.smem_stage = S::total;
+    v.smem_stage = kSmem;
     v.stage = &stage;
     v.step = &step;
     v.max_resident_blocks = &max_resident_blocks;
