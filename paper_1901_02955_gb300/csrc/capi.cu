@@ -555,6 +555,9 @@ static void tile_domains(std::vector<DomDev> &doms, const TileVariant &tv, int *
     D.tx = (D.nx + tv.tile[0] - 1) / tv.tile[0];
     D.ty = (D.ny + tv.tile[1] - 1) / tv.tile[1];
     D.tz = (D.nz + cz - 1) / cz;
+    const auto magic = [](int d) { return d > 1 ? unsigned((1ull << 32) / d) : 0xffffffffu; };
+    D.tx_magic = magic(D.tx);
+    D.ty_magic = magic(D.ty);
     D.tile_begin = prefix[i];
     prefix[i + 1] = prefix[i] + D.tx * D.ty * D.tz;
   }

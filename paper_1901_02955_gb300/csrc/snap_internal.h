@@ -60,6 +60,7 @@ struct DomDev {
   int tx, ty, tz;            // tiles per direction
   int tile_begin;            // first tile index of this domain in the launch
   int cz;                    // levels per tile
+  unsigned tx_magic, ty_magic;  // floor(2^32 / tx), floor(2^32 / ty), at most 2^32 - 1
   int bc[6];
   double dx, dy, dz;
   double grav, cfl, dt_fixed;

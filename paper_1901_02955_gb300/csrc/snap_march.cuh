@@ -18,53 +18,6 @@
 
 namespace snap {
 
-// What the march reads of its domain level by level, copied into shared memory once per tile (the
-// descriptor and the profiles in device memory cost two dependent loads per use): levels k0 ..
-// k0 + N - 1 of the profiles and the constants, under DomDev's names.
-template <class R, int N>
-struct Levels {
-  R x[N];
-  int k0;
-  __device__ __forceinline__ R operator[](int k) const { return x[k - k0]; }
-  __device__ __forceinline__ void fill(const R *from, int first, int end, int tid) {
-    if (tid == 0) k0 = first;
-    if (tid < N && first + tid >= 0 && first + tid < end) x[tid] = from[first + tid];
-  }
-};
-struct DomSides {
-  int bc[6];
-  double T_bot;
-  void *buf[3];  // the stage's input, Y^n and output at the tile's first cell of level 0
-};
-template <class R, int N>
-struct DomMarch;
-template <int N>
-struct DomMarch<float, N> : DomSides {
-  Levels<float, N> rb_hi, rb_lo, pc_f, pf_f, er_f, er_lo;
-  float fidx, fidy, fidz, fgrav;
-  __device__ __forceinline__ void fill(const DomDev &D, int first, int tid) {
-    rb_hi.fill(D.rb_hi, first, D.nz, tid);
-    rb_lo.fill(D.rb_lo, first, D.nz, tid);
-    pc_f.fill(D.pc_f, first, D.nz, tid);
-    pf_f.fill(D.pf_f, first, D.nz + 1, tid);
-    er_f.fill(D.er_f, first, D.nz, tid);
-    er_lo.fill(D.er_lo, first, D.nz, tid);
-    if (tid == 0) fidx = D.fidx, fidy = D.fidy, fidz = D.fidz, fgrav = D.fgrav;
-  }
-};
-template <int N>
-struct DomMarch<double, N> : DomSides {
-  Levels<double, N> rho_bar, p_cell, p_face, e_ref;
-  double idx, idy, idz, grav;
-  __device__ __forceinline__ void fill(const DomDev &D, int first, int tid) {
-    rho_bar.fill(D.rho_bar, first, D.nz, tid);
-    p_cell.fill(D.p_cell, first, D.nz, tid);
-    p_face.fill(D.p_face, first, D.nz + 1, tid);
-    e_ref.fill(D.e_ref, first, D.nz, tid);
-    if (tid == 0) idx = D.idx, idy = D.idy, idz = D.idz, grav = D.grav;
-  }
-};
-
 template <class R, class L, class T>
 struct MarchSmem {
   static constexpr int NC = T::TX * T::TY;
@@ -79,7 +32,7 @@ struct MarchSmem {
   static constexpr size_t e_off = bytes(NP), x_off = e_off + bytes(NE), q_off = x_off + bytes(NX);
   static constexpr size_t red_off = q_off + bytes(NC);
   static constexpr size_t dom_off = red_off + 32 * sizeof(double);
-  using Dom = DomMarch<R, T::TZ + 7>;  // levels z0 - 3 .. z0 + TZ + 3
+  using Dom = DomLocal<R, T::TZ + 7>;  // levels z0 - 3 .. z0 + TZ + 3
   static constexpr size_t total = dom_off + (sizeof(Dom) + 15) / 16 * 16;
   // location of (x, y) of the level whose rows start at cur: its row (a ragged tile's far y halo
   // lies in the rows it does not own), else the y halo
@@ -107,6 +60,8 @@ __device__ __forceinline__ void march_tiles(const StageArgs &a, const int stage,
   double *s_red = reinterpret_cast<double *>(smem + M::red_off);
   R *s_dt = reinterpret_cast<R *>(s_red + 31);  // the time step in the kernel's type
   typename M::Dom &S = *reinterpret_cast<typename M::Dom *>(smem + M::dom_off);
+  // the stage's input, Y^n and output at the tile's first column and level 0
+  void **s_buf = reinterpret_cast<void **>(s_red + 28);
   const Phys &ph = a.ph;
   const CstT<R> &C = cst<R>(a);
   const R weps = C.weno_eps;
@@ -119,19 +74,19 @@ __device__ __forceinline__ void march_tiles(const StageArgs &a, const int stage,
     const int nx = D.nx, ny = D.ny, nz = D.nz;
     const int lt = tile - D.tile_begin;
     const int cz = D.cz;  // levels per tile, at most T::TZ
-    const int x0 = (lt % D.tx) * TX, y0 = ((lt / D.tx) % D.ty) * TY, z0 = (lt / (D.tx * D.ty)) * cz;
+    int ix, iy, iz;
+    tile_coords(D, lt, ix, iy, iz);
+    const int x0 = ix * TX, y0 = iy * TY, z0 = iz * cz;
     const int ex = min(TX, nx - x0), ey = min(TY, ny - y0), ez = min(cz, nz - z0);
     const R *Ys = reinterpret_cast<const R *>(a.buf_s ? a.buf_s : D.buf[stage]);
-    double dt0 = 0.0;  // its loads are waited for after the columns' first levels
+    double dt0 = 0.0;  // waited for after the columns' first levels
     if (tid == 0) dt0 = stage_dt<RES>(a, D, stage, lt, s_red[0]);
     S.fill(D, z0 - 3, tid);
-    if (tid < 6) S.bc[tid] = D.bc[tid];
-    if (tid == 6) S.T_bot = D.T_bot;
     if (tid >= 8 && tid < 11) {
       const int i = tid - 8;  // input, Y^n, output
       const void *o = i == 0 ? a.buf_s : (i == 1 ? a.buf_n : a.buf_o);
       const int def = i == 0 ? stage : (i == 1 ? 0 : (stage + 1) % 3);
-      S.buf[i] = (R *)(o ? o : D.buf[def]) + ((long long)y0 * nx + x0);
+      s_buf[i] = (R *)(o ? o : D.buf[def]) + ((long long)y0 * nx + x0);
     }
     __syncthreads();
     const bool own = lx < ex && ly < ey;
@@ -158,10 +113,10 @@ __device__ __forceinline__ void march_tiles(const StageArgs &a, const int stage,
     const int hdir = tid < 6 * TX ? 1 : 0;
     if (has_h) hh = halo_cell<R>(a, D, stage, Ys, x0 + hx, y0 + hy, z0, hdir);
     const int hstep = has_h ? int(hh.stride / nz) : 0, plane = nx * ny;  // one level
-    const int at_col = ly * nx + lx;  // the thread's column from S.buf
+    const int at_col = ly * nx + lx;  // the thread's column from s_buf
     auto load_column = [&](int k) {  // the z sides are walls: beyond them the mirrored level
       const int gz = k < 0 ? -1 - k : (k >= nz ? 2 * nz - 1 - k : k);
-      load_fields<R, NV, RES>((const R *)S.buf[0] + ((long long)gz * plane + at_col),
+      load_fields<R, NV, RES>((const R *)s_buf[0] + ((long long)gz * plane + at_col),
                               (long long)plane * nz, yc);
     };
     auto store_column = [&](int k, int slot) {
@@ -310,8 +265,8 @@ __device__ __forceinline__ void march_tiles(const StageArgs &a, const int stage,
       const long long g = (long long)k * plane + at_col, ncell = (long long)plane * nz;
       R ys[NV], yn[NV];
       if (own) {
-        load_fields<R, NV, RES>((const R *)S.buf[0] + g, ncell, ys);
-        if (stage != 0) load_fields<R, NV, RES>((const R *)S.buf[1] + g, ncell, yn);
+        load_fields<R, NV, RES>((const R *)s_buf[0] + g, ncell, ys);
+        if (stage != 0) load_fields<R, NV, RES>((const R *)s_buf[1] + g, ncell, yn);
       }
       __syncthreads();
       // ---- D. divergence, sources, stage combine, store; the loads of the next round go first
@@ -341,7 +296,7 @@ __device__ __forceinline__ void march_tiles(const StageArgs &a, const int stage,
         }
         finish_cell<R, L, MICRO>(a, S, ph, C, stage, dt, k, ys, acc, mb, mt,
                                  [&](int v) { return yn[v]; }, yo);
-        R *out = (R *)S.buf[2] + g;
+        R *out = (R *)s_buf[2] + g;
 #pragma unroll
         for (int v = 0; v < NV; ++v, out += ncell) *out = yo[v];
         if (stage == 2)

@@ -263,6 +263,73 @@ struct SV {
   }
 };
 
+// What a tile's inner loops read of their domain, copied into shared memory once per tile (the
+// descriptor and the profiles in device memory cost two dependent loads per use): levels k0 ..
+// k0 + N - 1 of the profiles and the constants, under DomDev's names.
+template <class R, int N>
+struct Levels {
+  R x[N];
+  int k0;
+  __device__ __forceinline__ R operator[](int k) const { return x[k - k0]; }
+  // by one warp
+  __device__ __forceinline__ void fill(const R *from, int first, int end, int lane) {
+    if (lane == 0) k0 = first;
+    for (int i = lane; i < N; i += 32)
+      if (first + i >= 0 && first + i < end) x[i] = from[first + i];
+  }
+};
+struct DomSides {
+  int bc[6];
+  double T_bot;
+  __device__ __forceinline__ void fill_sides(const DomDev &D, int lane) {
+    if (lane < 6) bc[lane] = D.bc[lane];
+    if (lane == 6) T_bot = D.T_bot;
+  }
+};
+// fill: the CTA's first four warps, a profile or two each
+template <class R, int N>
+struct DomLocal;
+template <int N>
+struct DomLocal<float, N> : DomSides {
+  Levels<float, N> rb_hi, rb_lo, pc_f, pf_f, er_f, er_lo;
+  float fidx, fidy, fidz, fgrav;
+  __device__ __forceinline__ void fill(const DomDev &D, int first, int tid) {
+    const int lane = tid & 31;
+    if (tid < 32) {
+      fill_sides(D, lane);
+      rb_hi.fill(D.rb_hi, first, D.nz, lane);
+    } else if (tid < 64) {
+      rb_lo.fill(D.rb_lo, first, D.nz, lane);
+      pc_f.fill(D.pc_f, first, D.nz, lane);
+    } else if (tid < 96) {
+      pf_f.fill(D.pf_f, first, D.nz + 1, lane);
+      er_f.fill(D.er_f, first, D.nz, lane);
+    } else if (tid < 128) {
+      er_lo.fill(D.er_lo, first, D.nz, lane);
+      if (lane == 0) fidx = D.fidx, fidy = D.fidy, fidz = D.fidz, fgrav = D.fgrav;
+    }
+  }
+};
+template <int N>
+struct DomLocal<double, N> : DomSides {
+  Levels<double, N> rho_bar, p_cell, p_face, e_ref;
+  double idx, idy, idz, grav;
+  __device__ __forceinline__ void fill(const DomDev &D, int first, int tid) {
+    const int lane = tid & 31;
+    if (tid < 32) {
+      fill_sides(D, lane);
+      rho_bar.fill(D.rho_bar, first, D.nz, lane);
+    } else if (tid < 64) {
+      p_cell.fill(D.p_cell, first, D.nz, lane);
+    } else if (tid < 96) {
+      p_face.fill(D.p_face, first, D.nz + 1, lane);
+    } else if (tid < 128) {
+      e_ref.fill(D.e_ref, first, D.nz, lane);
+      if (lane == 0) idx = D.idx, idy = D.idy, idz = D.idz, grav = D.grav;
+    }
+  }
+};
+
 // Per-level reference values in the kernel's type: FP32 kernels read FP32 copies, FP64
 // kernels the FP64 originals. DD is DomDev, or a kernel's own copy of what it needs of it.
 template <class R>
@@ -758,16 +825,37 @@ __device__ __forceinline__ int map_index(int g, int n, int bc_lo, int bc_hi, boo
   return g;
 }
 
+// The domain of a tile: the last whose first tile is not beyond it. Every lane of a warp takes part:
+// 32 candidates per round, so two dependent loads for up to 1024 domains (a binary search by
+// every thread took log2 of them: 7 for the 96-domain ensemble, before anything else of the tile
+// could start).
 __device__ __forceinline__ int find_domain(const int *prefix, int ndom, int tile) {
-  int lo = 0, hi = ndom - 1;
-  while (lo < hi) {
-    int mid = (lo + hi + 1) >> 1;
-    if (__ldg(prefix + mid) <= tile)
-      lo = mid;
-    else
-      hi = mid - 1;
+  int lo = 0, n = ndom;  // the answer is one of lo .. lo + n - 1
+  while (n > 1) {
+    const int step = (n + 31) / 32, i = int(threadIdx.x & 31) * step;
+    const bool ok = i < n && __ldg(prefix + lo + i) <= tile;
+    const int c = (31 - __clz(__ballot_sync(0xffffffffu, ok))) * step;  // lane 0's test holds
+    lo += c;
+    n = min(step, n - c);
   }
   return lo;
+}
+
+// n / d and n % d for n >= 0 by the precomputed floor(2^32 / d): the high product is the quotient
+// or one less
+__device__ __forceinline__ void divide(int n, int d, unsigned magic, int &quot, int &rem) {
+  quot = int(__umulhi(unsigned(n), magic));
+  rem = n - quot * d;
+  if (rem >= d) {
+    ++quot;
+    rem -= d;
+  }
+}
+// Tile coordinates of tile lt of a domain.
+__device__ __forceinline__ void tile_coords(const DomDev &D, int lt, int &ix, int &iy, int &iz) {
+  int q;
+  divide(lt, D.tx, D.tx_magic, q, ix);
+  divide(q, D.ty, D.ty_magic, iz, iy);
 }
 
 __device__ __forceinline__ double block_max(double v, double *red) {
@@ -1057,11 +1145,12 @@ __device__ __forceinline__ void weno5_pair(R a, R b, R c, R d, R e, R eps, R &qm
   // instantiation rounds the same way whatever its register allocation
   using A = Ar<R>;
   constexpr R k3 = R(3.0 / 13.0);
-  const R u = c - b, v = d - c, w = b - a, z = e - d;
-  const R s0 = u - w, s1 = v - u, s2 = z - v;
-  const R r0 = A::fma_(R(2), u, s0);   // a - 4b + 3c
-  const R r1 = u + v;                  // d - b
-  const R r2 = A::fma_(R(-2), v, s2);  // 3c - 4d + e
+  // (w, z, s2 and r2 with the opposite signs)
+  const R u = c - b, v = d - c, w = a - b, z = d - e;
+  const R s0 = u + w, s1 = v - u, s2 = v + z;
+  const R r0 = A::fma_(R(3), u, w);  // a - 4b + 3c
+  const R r1 = u + v;                // d - b
+  const R r2 = A::fma_(R(3), v, z);  // -(3c - 4d + e)
   eps *= R(12.0 / 13.0);
   const R e0 = A::fma_(k3 * r0, r0, A::fma_(s0, s0, eps));
   const R e1 = A::fma_(k3 * r1, r1, A::fma_(s1, s1, eps));
@@ -1087,13 +1176,13 @@ __device__ __forceinline__ void weno5_pair(R a, R b, R c, R d, R e, R eps, R &qm
   const R Sp = A::fma_(R(3), g0, A::fma_(R(6), g1, g2));
   // the bracketed sums, -(g0 D1 / 3 + g2 D2 / 2) and g0 D1 / 2 + g2 D2 / 3, from the halves of
   // the third differences (signs chosen so that no operand needs a negation, which the packed
-  // instructions of weno5_pair2 do not have)
+  // instructions of weno5_pair2 do not have, and few constants, which take them a register pair each)
   const R h1 = R(0.5) * s1;
   const R P = g0 * A::fma_(R(-0.5), s0, h1);  // g0 D1 / 2
-  const R Q = g2 * A::fma_(R(-0.5), s2, h1);  // -g2 D2 / 2
+  const R Q = g2 * A::fma_(R(0.5), s2, h1);   // -g2 D2 / 2
   const R Nm = A::fma_(R(-2.0 / 3.0), P, Q);
   const R Np = A::fma_(R(-2.0 / 3.0), Q, P);
-  const R cm = A::fma_(R(1.0 / 6.0), A::fma_(R(2), v, u), c);
+  const R cm = A::fma_(R(1.0 / 6.0), r1 + v, c);
   const R cp = A::fma_(R(-0.5), r1, cm);  // c - (v + 2 u) / 6
   if constexpr (sizeof(R) == 8) {
     // 1/Sm = Sp / (Sm Sp) and 1/Sp = Sm / (Sm Sp); one division each only if the product
@@ -1124,13 +1213,12 @@ __device__ __forceinline__ void weno5_pair2(float2 a, float2 b, float2 c, float2
   // the operations of weno5_pair in the same order (differences as fused multiply-adds by -1,
   // which round the same)
   const float2 k3 = f2c(3.0f / 13.0f), m1f = f2c(-1.0f);
-  const float2 u = __ffma2_rn(m1f, b, c), v = __ffma2_rn(m1f, c, d), w = __ffma2_rn(m1f, a, b),
-               z = __ffma2_rn(m1f, d, e);
-  const float2 s0 = __ffma2_rn(m1f, w, u), s1 = __ffma2_rn(m1f, u, v),
-               s2 = __ffma2_rn(m1f, v, z);
-  const float2 r0 = __ffma2_rn(f2c(2.0f), u, s0);   // a - 4b + 3c
-  const float2 r1 = __fadd2_rn(u, v);               // d - b
-  const float2 r2 = __ffma2_rn(f2c(-2.0f), v, s2);  // 3c - 4d + e
+  const float2 u = __ffma2_rn(m1f, b, c), v = __ffma2_rn(m1f, c, d), w = __ffma2_rn(m1f, b, a),
+               z = __ffma2_rn(m1f, e, d);
+  const float2 s0 = __fadd2_rn(u, w), s1 = __ffma2_rn(m1f, u, v), s2 = __fadd2_rn(v, z);
+  const float2 r0 = __ffma2_rn(f2c(3.0f), u, w);
+  const float2 r1 = __fadd2_rn(u, v);
+  const float2 r2 = __ffma2_rn(f2c(3.0f), v, z);
   const float2 ke = f2c(eps * (12.0f / 13.0f));
   const float2 e0 = __ffma2_rn(__fmul2_rn(k3, r0), r0, __ffma2_rn(s0, s0, ke));
   const float2 e1 = __ffma2_rn(__fmul2_rn(k3, r1), r1, __ffma2_rn(s1, s1, ke));
@@ -1143,10 +1231,10 @@ __device__ __forceinline__ void weno5_pair2(float2 a, float2 b, float2 c, float2
   const float2 Sp = __ffma2_rn(f2c(3.0f), g0, __ffma2_rn(f2c(6.0f), g1, g2));
   const float2 h1 = __fmul2_rn(f2c(0.5f), s1);
   const float2 P = __fmul2_rn(g0, __ffma2_rn(f2c(-0.5f), s0, h1));
-  const float2 Q = __fmul2_rn(g2, __ffma2_rn(f2c(-0.5f), s2, h1));
+  const float2 Q = __fmul2_rn(g2, __ffma2_rn(f2c(0.5f), s2, h1));
   const float2 Nm = __ffma2_rn(f2c(-2.0f / 3.0f), P, Q);
   const float2 Np = __ffma2_rn(f2c(-2.0f / 3.0f), Q, P);
-  const float2 cm = __ffma2_rn(f2c(1.0f / 6.0f), __ffma2_rn(f2c(2.0f), v, u), c);
+  const float2 cm = __ffma2_rn(f2c(1.0f / 6.0f), __fadd2_rn(r1, v), c);
   const float2 cp = __ffma2_rn(f2c(-0.5f), r1, cm);
   qm = __ffma2_rn(Nm, f2rcp(Sm), cm);
   qp = __ffma2_rn(Np, f2rcp(Sp), cp);
@@ -1432,7 +1520,28 @@ __device__ __forceinline__ void finish_cell(const StageArgs &a, const DD &D, con
   if (!(rs > R(0)) || !isfinite(yo[L::IE])) atomicOr(a.flags, (unsigned)kFlagNonFinite);
 }
 
-// One stage over the CTA's tiles. RES (the resident step, one tile per CTA for all three
+// Viscous flux of one face (Sec. 5.1), added to F: -rho_f nu du/dn and -rho_f nu (u_f du/dn + c_pd
+// Pi_f dtheta/dn) between the cells at locations bl and br, with the face means as halves of
+// sums: k = rho_f nu / dn. ih: inverse cell size along the face's normal.
+template <class R, class L>
+__device__ __forceinline__ void viscous_flux(const CstT<R> &C, R ih, const R *prim, const R *th,
+                                             const R *pi, int bl, int br, int N, R *F) {
+  using V = SV<R, L::NV>;
+  R XL[L::NV], XR[L::NV];
+  V::load(prim, bl, N, XL);
+  V::load(prim, br, N, XR);
+  const R k = (XL[0] + XR[0]) * (R(0.5) * C.nu * ih);
+  R w2 = (C.c_pd * (pi[bl] + pi[br])) * (th[br] - th[bl]);
+#pragma unroll
+  for (int m = L::IM0; m < L::IM0 + L::NMOM; ++m) {
+    const R du = XR[m] - XL[m];
+    F[m] = Ar<R>::fma_(-k, du, F[m]);
+    w2 = Ar<R>::fma_(XL[m] + XR[m], du, w2);
+  }
+  F[L::IE] = Ar<R>::fma_(R(-0.5) * k, w2, F[L::IE]);
+}
+
+// One stage over the CTA's 3-D one-shot tiles. RES (the resident step, one tile per CTA for all three
 // stages): for stages 1 and 2 ys holds the owned cells' stage input on entry (the previous
 // stage's output, kept in registers) instead of being loaded; Y^n of the owned cells is kept
 // in shared memory from stage 0 on; the time step of stage 0 stays in s_red[0]; ghost cells
@@ -1443,6 +1552,7 @@ template <class R, class L, bool VISC, class T, bool MICRO, bool RES = false>
 __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
                                             unsigned char *smem,
                                             R (&ys)[Box<T, L::D3>::CPT][L::NV]) {
+  static_assert(L::D3, "the x-z plane has its own kernel (plane_tiles)");
   using B = Box<T, L::D3>;
   using S = StageSmem<R, L, VISC, T>;
   using P = Prof<R>;
@@ -1467,9 +1577,9 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
     const int nx = D.nx, ny = D.ny, nz = D.nz;
     const long long ncell = D.ncell;
     const int lt = tile - D.tile_begin;
-    const int x0 = (lt % D.tx) * TX;
-    const int y0 = ((lt / D.tx) % D.ty) * TY;
-    const int z0 = (lt / (D.tx * D.ty)) * TZ;
+    int ix, iy, iz;
+    tile_coords(D, lt, ix, iy, iz);
+    const int x0 = ix * TX, y0 = iy * TY, z0 = iz * TZ;
     const int ex = min(TX, nx - x0), ey = min(TY, ny - y0), ez = min(TZ, nz - z0);
     const R *Ys = reinterpret_cast<const R *>(a.buf_s ? a.buf_s : D.buf[stage]);
     const R *Yn = reinterpret_cast<const R *>(a.buf_n ? a.buf_n : D.buf[0]);
@@ -1521,7 +1631,7 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
     }
     // ---- 2. halo of the cross (x, y, z), boundary ghosts synthesised --------------------
     {
-      constexpr int NHX = 6 * TY * TZ, NHY = L::D3 ? 6 * TX * TZ : 0, NHZ = 6 * TX * TY;
+      constexpr int NHX = 6 * TY * TZ, NHY = 6 * TX * TZ, NHZ = 6 * TX * TY;
       for (int h = tid; h < NHX + NHY + NHZ; h += NT) {
         int bx, by, bz, dirn, layer;
         bool ok;
@@ -1581,17 +1691,15 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
     // ---- 3. per direction: WENO5 per cell (both faces), LMARS per face, divergence -------
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      if (d == 1 && !L::D3) continue;
       const int fx = d == 0, fy = d == 1, fz = d == 2;
       // face array strides: faces along d are numbered 0..T_d
       const int sx = TX + fx, sy = TY + fy;
-      const int stride = d == 0 ? 1 : (d == 1 ? B::BX : B::BX * B::BY);
       const int ed = d == 0 ? ex : (d == 1 ? ey : ez);
       // 3a. reconstruction over the owned cells and one more on each side along d
       {
         const int rx = TX + 2 * fx, ry = TY + 2 * fy, rz = TZ + 2 * fz;
         const int nrec = rx * ry * rz;
-        constexpr int MAXREC = (TX + 2) * (TY + (L::D3 ? 2 : 0)) * (TZ + 2);
+        constexpr int MAXREC = (TX + 2) * (TY + 2) * (TZ + 2);
 #pragma unroll
         for (int r = 0; r < (MAXREC + NT - 1) / NT; ++r) {
           const int it = tid + r * NT;
@@ -1601,10 +1709,10 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
           lz -= fz;
           const int ld = fx ? lx : (fy ? ly : lz);
           if (it < nrec && ld <= ed && lx < ex + fx && ly < ey + fy && lz < ez + fz) {
-            // the five cells of the window along d: a fixed stride in the x-z box and along the
-            // 3-D x-lines; mapped one by one where a 3-D y or z window leaves the x-lines
+            // the five cells of the window along d: unit stride along the x-lines, mapped one by
+            // one where a y or z window leaves them
             int o[5];
-            if (L::D3 && !fx) {
+            if (!fx) {
               // the window's fixed coordinate lies in the owned range
 #pragma unroll
               for (int k = 0; k < 5; ++k)
@@ -1613,7 +1721,7 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
             } else {
               const int bi = B::idx(lx + 3, ly + B::HY, lz + 3);
 #pragma unroll
-              for (int k = 0; k < 5; ++k) o[k] = bi + (k - 2) * stride;
+              for (int k = 0; k < 5; ++k) o[k] = bi + k - 2;
             }
             const int fl = ((lz + fz) * sy + (ly + fy)) * sx + (lx + fx);  // face c+1/2
             const int fr = (lz * sy + ly) * sx + lx;                        // face c-1/2
@@ -1649,20 +1757,7 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
           if constexpr (VISC) {
             const int bi = B::idx(ix + 3, iy + B::HY, iz + 3);  // right cell of the face
             const int bl = B::idx(ix + 3 - fx, iy + B::HY - fy, iz + 3 - fz);
-            R XLc[NV], XRc[NV];  // primitives of the two cells of the face
-            V::load(s_prim, bl, B::NSTORE, XLc);
-            V::load(s_prim, bi, B::NSTORE, XRc);
-            // -rho_f nu du/dn and -rho_f nu (u_f du/dn + c_pd Pi_f dtheta/dn) with the face
-            // means as halves of sums: k = rho_f nu / dn
-            const R k = (XLc[0] + XRc[0]) * (R(0.5) * C.nu * P::ih(D, d));
-            R w2 = (C.c_pd * (s_pi[bl] + s_pi[bi])) * (s_th[bi] - s_th[bl]);
-#pragma unroll
-            for (int mm = 0; mm < L::NMOM; ++mm) {
-              const R ul = XLc[L::IM0 + mm], ur = XRc[L::IM0 + mm], du = ur - ul;
-              F[L::IM0 + mm] = Ar<R>::fma_(-k, du, F[L::IM0 + mm]);
-              w2 = Ar<R>::fma_(ul + ur, du, w2);
-            }
-            F[L::IE] = Ar<R>::fma_(R(-0.5) * k, w2, F[L::IE]);
+            viscous_flux<R, L>(C, P::ih(D, d), s_prim, s_th, s_pi, bl, bi, B::NSTORE, F);
           }
           V::store(s_fl, f, B::NF, F);
         }
@@ -1736,6 +1831,358 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
   }
 }
 
+// ------------------------------------------------------------------------------------------
+// the x-z plane
+// ------------------------------------------------------------------------------------------
+// Shared memory of an x-z tile: the boxed primitives (and theta, Exner function), per direction
+// the left states of its faces, overwritten by their fluxes, the right states of the far x
+// faces, the local copy of the domain, and Y^n of the owned cells where that costs no resident
+// CTA (228 KB of shared memory per SM, 1 KB reserved per CTA).
+template <class R, class L, bool VISC, class T>
+struct PlaneSmem {
+  using B = Box<T, false>;
+  static constexpr int RPB = T::NT / T::TX;                     // rows per round of the CTA
+  static constexpr int M = (T::TZ + 2 + RPB - 1) / RPB;         // rounds over rows -1 .. TZ
+  static constexpr int NX = (T::TX + 1) * T::TZ, NZ = T::TX * (T::TZ + 1);
+  static constexpr int NEXTRA = 4 * T::TX + 6 * T::TZ;          // halo cells outside those rows
+  static constexpr size_t bytes(int n, int nv) { return (sizeof(R) * nv * n + 15) / 16 * 16; }
+  static constexpr size_t visc_off = bytes(B::NBOX, L::NV);
+  static constexpr size_t x_off = visc_off + (VISC ? bytes(B::NBOX, 2) : 0);
+  static constexpr size_t z_off = x_off + bytes(NX, L::NV);
+  static constexpr size_t r_off = z_off + bytes(NZ, L::NV);
+  static constexpr size_t red_off = r_off + bytes(T::TZ, L::NV);
+  static constexpr size_t dom_off = red_off + 32 * sizeof(double);
+  using Dom = DomLocal<R, T::TZ + 7>;  // levels z0 - 3 .. z0 + TZ + 3
+  // both directions in the same phases (three barriers instead of five) where their states fit
+  // the registers: the four dry fields (5 % of the FP32 step), not the seven moist ones
+  static constexpr bool BOTH = L::NV <= 4;
+  static constexpr size_t base = dom_off + (sizeof(Dom) + 15) / 16 * 16;
+  static constexpr size_t yn_bytes = sizeof(R) * L::NV * T::NT * M;
+  static constexpr bool PREFETCH = 233472 / (base + yn_bytes + 1024) >= 233472 / (base + 1024);
+  static constexpr size_t total = base + (PREFETCH ? yn_bytes : 0);
+};
+
+// One stage over the CTA's x-z tiles. A thread keeps column lx = tid mod TX of rows row, row + RPB,
+// .. (row -1 and row ez are the z halo next to the tile, reconstructed for the outer z faces): it
+// converts these cells, reconstructs them, solves the face on their lower side from its own right
+// state (kept in registers) and its neighbour's left state (shared memory), and finishes them
+// with its own lower flux and the neighbour's. Rounds, rows and columns are powers of two or
+// constants, so an item's locations are the thread's plus an immediate. RES as for stage_tiles.
+//
+// Bound by instruction issue (FP32) and the FP64 pipe (FP64). All loads of a tile go out together,
+// then the domain's profiles, then the conversions; dividing item numbers into rows and columns,
+// reading the profiles through the descriptor and exchanging both states of every face through
+// shared memory took 911 instructions per cell where this takes 826 (density current 1024 x 256,
+// FP32: 38.6 -> 35.8 us per step; 96-domain ensemble 1.83 -> 1.74 ms, one moist bubble of 61 x 47
+// cells 31.9 -> 29 us). Four cells per thread instead of two at the same tile are slower (39.5
+// us; ensemble 2.16 ms): the warps are what hides the phases' latency.
+template <class R, class L, bool VISC, class T, bool MICRO, bool RES = false>
+__device__ __forceinline__ void plane_tiles(const StageArgs &a, const int stage,
+                                            unsigned char *smem,
+                                            R (&ys)[PlaneSmem<R, L, VISC, T>::M][L::NV]) {
+  using S = PlaneSmem<R, L, VISC, T>;
+  using B = Box<T, false>;
+  using P = Prof<R>;
+  using V = SV<R, L::NV>;
+  constexpr int NV = L::NV, TX = T::TX, TZ = T::TZ, NT = T::NT, M = S::M, RPB = S::RPB;
+  constexpr int BX = B::BX, NB = B::NBOX, NE = (S::NEXTRA + NT - 1) / NT;
+  static_assert((TX & (TX - 1)) == 0 && NT % TX == 0 && 2 * TZ <= NT && NT >= 128, "columns of whole rounds");
+  R *s_prim = reinterpret_cast<R *>(smem);
+  R *s_th = reinterpret_cast<R *>(smem + S::visc_off), *s_pi = s_th + (VISC ? NB : 0);
+  R *s_x = reinterpret_cast<R *>(smem + S::x_off), *s_z = reinterpret_cast<R *>(smem + S::z_off);
+  R *s_r = reinterpret_cast<R *>(smem + S::r_off);
+  double *s_red = reinterpret_cast<double *>(smem + S::red_off);
+  R *s_dt = reinterpret_cast<R *>(s_red + 31);
+  typename S::Dom &Dl = *reinterpret_cast<typename S::Dom *>(smem + S::dom_off);
+  R *s_yn = reinterpret_cast<R *>(smem + S::base);  // used when S::PREFETCH
+  const Phys &ph = a.ph;
+  const CstT<R> &C = cst<R>(a);
+  const R weps = C.weno_eps;
+  const int tid = threadIdx.x, lx = tid % TX, row = tid / TX;
+  const int bi0 = (row + 2) * BX + lx + 3;  // the thread's cell of round 0 (row row - 1)
+
+  for (int tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
+    const int dm = find_domain(a.tile_domain, a.ndom, tile);
+    const DomDev &D = a.doms[dm];
+    const int nx = D.nx, nz = D.nz;
+    const long long ncell = D.ncell;
+    const int lt = tile - D.tile_begin;
+    int ix, iz;
+    divide(lt, D.tx, D.tx_magic, iz, ix);
+    const int x0 = ix * TX, z0 = iz * TZ;
+    const int ex = min(TX, nx - x0), ez = min(TZ, nz - z0);
+    const R *Ys = reinterpret_cast<const R *>(a.buf_s ? a.buf_s : D.buf[stage]);
+    const R *Yn = reinterpret_cast<const R *>(a.buf_n ? a.buf_n : D.buf[0]);
+    R *Yo = reinterpret_cast<R *>(a.buf_o ? a.buf_o : D.buf[stage == 0 ? 1 : (stage == 1 ? 2 : 0)]);
+    auto level = [&](int r) {  // row r's level, mirrored at the z walls
+      const int k = z0 + r;
+      return k < 0 ? -1 - k : (k >= nz ? 2 * nz - 1 - k : k);
+    };
+    auto owned = [&](int m) { return lx < ex && (unsigned)(row + m * RPB - 1) < (unsigned)ez; };
+    // ---- 1. every load of the tile, then the local copy of the domain, then the conversions
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const int r = row + m * RPB - 1;
+      if (lx < ex && r <= ez && !(RES && stage > 0 && owned(m)))
+        load_fields<R, NV, RES>(Ys + ((long long)level(r) * nx + (x0 + lx)), ncell, ys[m]);
+    }
+    // the halo cells outside rows -1 .. ez: four z rows, then three columns on each x side
+    HaloCell<R> hc[NE];
+    R yh[NE][NV];
+    int hb[NE];  // box location, -1: none
+    bool hx[NE];
+#pragma unroll
+    for (int e = 0; e < NE; ++e) {
+      const int h = tid + e * NT;
+      hb[e] = -1;
+      hx[e] = h >= 4 * TX;
+      int x = 0, r = 0;
+      bool ok = false;
+      if (!hx[e]) {
+        const int q = h / TX;
+        x = h % TX;
+        r = q < 2 ? q - 3 : ez + q - 1;
+        ok = x < ex;
+      } else if (h < S::NEXTRA) {
+        const int q = (h - 4 * TX) % 6;
+        r = (h - 4 * TX) / 6;
+        x = q < 3 ? q - 3 : ex + q - 3;
+        ok = r < ez;
+      }
+      if (ok) {
+        hb[e] = (r + 3) * BX + x + 3;
+        if (hx[e])
+          hc[e] = halo_cell<R>(a, D, stage, Ys, x0 + x, 0, z0 + r, 0);
+        else
+          hc[e] = halo_cell<R>(a, D, stage, Ys, x0 + x, 0, z0 + r, 2);
+        load_fields<R, NV, RES>(hc[e].src, hc[e].stride, yh[e]);
+      }
+    }
+    if constexpr (S::PREFETCH && !RES) {
+      if (stage != 0) {
+#pragma unroll
+        for (int m = 0; m < M; ++m)
+          if (owned(m)) {
+            const R *src = Yn + ((long long)(z0 + row + m * RPB - 1) * nx + (x0 + lx));
+#pragma unroll
+            for (int v = 0; v < NV; ++v)
+              cp_async_elem<R>(s_yn + (m * NV + v) * NT + tid, src + v * ncell);
+          }
+        cp_async_commit();
+      }
+    }
+    Dl.fill(D, z0 - 3, tid);
+    if (tid == NT - 1) {  // while the tile's loads are on their way
+      const double dt = stage_dt<RES>(a, D, stage, lt, s_red[0]);
+      s_red[0] = dt;
+      *s_dt = R(dt);
+    }
+    __syncthreads();
+    auto store_prim = [&](const R *x, R pt, int b, bool heat) {
+      V::store(s_prim, b, NB, x);
+      // the viscous heat flux reads theta and the Exner function only on the two sides of a
+      // face: not beyond the ring next to the tile
+      if constexpr (VISC) {
+        if (heat) {
+          const R Pi = Ar<R>::pow_small(pt * R(1e-5), C.kappa);
+          s_th[b] = pt * Ar<R>::rcp(x[0] * Pi) * C.iR_d;
+          s_pi[b] = Pi;
+        }
+      }
+    };
+#pragma unroll
+    for (int m = 0; m < M; ++m) {
+      const int r = row + m * RPB - 1;
+      if (lx < ex && r <= ez) {
+        HaloCell<R> c;
+        c.gz = level(r);
+        c.flip = c.gz != z0 + r;
+        c.side = z0 + r < 0 ? 4 : 5;
+        R x[NV], pt;
+        halo_prim<R, L>(Dl, ph, C, c, 2, ys[m], x, pt);
+        store_prim(x, pt, bi0 + m * RPB * BX, true);
+        if constexpr (RES && S::PREFETCH) {
+          if (stage == 0) {
+#pragma unroll
+            for (int v = 0; v < NV; ++v) s_yn[(m * NV + v) * NT + tid] = ys[m][v];
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < NE; ++e)
+      if (hb[e] >= 0) {
+        R x[NV], pt;
+        halo_prim<R, L>(Dl, ph, C, hc[e], hx[e] ? 0 : 2, yh[e], x, pt);
+        const int q = (tid + e * NT - 4 * TX) % 6;
+        store_prim(x, pt, hb[e], hx[e] && (q == 2 || q == 3));
+      }
+    __syncthreads();
+
+    // ---- 2. per direction: states, face fluxes (over the left states), divergence. Qx, Qz: the
+    // right state of the cell's lower face, then that face's flux. x: the owned cells, and the
+    // column on either side by the threads whose last row lies above the tile
+    R acc[M][NV], Q[S::BOTH ? 2 : 1][M][NV];
+    auto &Qx = Q[0], &Qz = Q[S::BOTH ? 1 : 0];
+    const int e = NT - 1 - tid;  // the last threads first
+    auto x_states = [&]() {
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if (owned(m)) {
+          const int r = row + m * RPB - 1, b = bi0 + m * RPB * BX;
+          const int o[5] = {b - 2, b - 1, b, b + 1, b + 2};
+          R QM[NV];
+          recon_window<R, NV>(s_prim, o, NB, weps, QM, Qx[m]);
+          V::store(s_x, r * (TX + 1) + lx + 1, S::NX, QM);
+        }
+      if (e < 2 * TZ) {
+        const int r = e >> 1;
+        const bool far = e & 1;
+        if (r < ez) {
+          const int b = (r + 3) * BX + (far ? ex : -1) + 3;
+          const int o[5] = {b - 2, b - 1, b, b + 1, b + 2};
+          R QM[NV], QP[NV];
+          recon_window<R, NV>(s_prim, o, NB, weps, QM, QP);
+          if (far)
+            V::store(s_r, r, TZ, QP);
+          else
+            V::store(s_x, r * (TX + 1), S::NX, QM);
+        }
+      }
+    };
+    auto x_fluxes = [&]() {
+#pragma unroll
+      for (int m = 0; m < M; ++m)
+        if (owned(m)) {
+          const int r = row + m * RPB - 1, f = r * (TX + 1) + lx, b = bi0 + m * RPB * BX;
+          R QL[NV], F[NV];
+          V::load(s_x, f, S::NX, QL);
+          lmars<R, L>(C, QL, Qx[m], 0, P::pc(Dl, z0 + r), F);
+          if constexpr (VISC)
+            viscous_flux<R, L>(C, P::ih(Dl, 0), s_prim, s_th, s_pi, b - 1, b, NB, F);
+          V::store(s_x, f, S::NX, F);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) Qx[m][v] = F[v];
+        }
+      if (e < TZ && e < ez) {
+        const int f = e * (TX + 1) + ex, b = (e + 3) * BX + ex + 3;
+        R QL[NV], QR[NV], F[NV];
+        V::load(s_x, f, S::NX, QL);
+        V::load(s_r, e, TZ, QR);
+        lmars<R, L>(C, QL, QR, 0, P::pc(Dl, z0 + e), F);
+        if constexpr (VISC)
+          viscous_flux<R, L>(C, P::ih(Dl, 0), s_prim, s_th, s_pi, b - 1, b, NB, F);
+        V::store(s_x, f, S::NX, F);
+      }
+    };
+    auto x_divergence = [&](int m) {
+      if (owned(m)) {
+        R F1[NV];
+        V::load(s_x, (row + m * RPB - 1) * (TX + 1) + lx + 1, S::NX, F1);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) acc[m][v] = -((F1[v] - Qx[m][v]) * P::ih(Dl, 0));
+      }
+    };
+    auto z_states = [&](int m) {
+      const int r = row + m * RPB - 1, b = bi0 + m * RPB * BX;
+      if (lx < ex && r <= ez) {
+        const int o[5] = {b - 2 * BX, b - BX, b, b + BX, b + 2 * BX};
+        R QM[NV];
+        recon_window<R, NV>(s_prim, o, NB, weps, QM, Qz[m]);
+        if (r < ez) V::store(s_z, (r + 1) * TX + lx, S::NZ, QM);
+      }
+    };
+    auto z_fluxes = [&]() {
+#pragma unroll
+      for (int m = 0; m < M; ++m) {
+        const int r = row + m * RPB - 1, f = r * TX + lx, b = bi0 + m * RPB * BX, kf = z0 + r;
+        if (lx < ex && r >= 0 && r <= ez) {
+          R QL[NV], F[NV];
+          V::load(s_z, f, S::NZ, QL);
+          const R pref = P::pf(Dl, kf);
+          lmars<R, L>(C, QL, Qz[m], 2, pref, F);
+          if constexpr (L::MOIST && MICRO) {
+            // no condensate passes a wall
+            if (ph.sediment && !(kf == 0 && Dl.bc[4] != kBcPeriodic) &&
+                !(kf == nz && Dl.bc[5] != kBcPeriodic))
+              sediment_flux<R, L>(C, QL, Qz[m], pref, F);
+          }
+          if constexpr (VISC)
+            viscous_flux<R, L>(C, P::ih(Dl, 2), s_prim, s_th, s_pi, b - BX, b, NB, F);
+          V::store(s_z, f, S::NZ, F);
+#pragma unroll
+          for (int v = 0; v < NV; ++v) Qz[m][v] = F[v];
+        }
+      }
+    };
+    if constexpr (S::BOTH) {
+      x_states();
+#pragma unroll
+      for (int m = 0; m < M; ++m) z_states(m);
+      __syncthreads();
+      x_fluxes();
+      z_fluxes();
+    } else {
+      x_states();
+      __syncthreads();
+      x_fluxes();
+      __syncthreads();
+#pragma unroll
+      for (int m = 0; m < M; ++m) {  // the face arrays of the two directions are separate
+        x_divergence(m);
+        z_states(m);
+      }
+      __syncthreads();
+      z_fluxes();
+    }
+    if constexpr (S::PREFETCH && !RES) {
+      if (stage != 0) cp_async_wait();  // this thread's own copies of Y^n
+    }
+    __syncthreads();
+    const R dt = *s_dt;
+
+    // ---- 3. z divergence, gravity source, stage combine, saturation adjustment, store
+    R rate_max = R(0);
+#pragma unroll
+    for (int m = 0; m < M; ++m)
+      if (owned(m)) {
+        const int r = row + m * RPB - 1, k = z0 + r;
+        if constexpr (S::BOTH) x_divergence(m);
+        R F1[NV], yo[NV], mb = R(0), mt = R(0);
+        V::load(s_z, (r + 1) * TX + lx, S::NZ, F1);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+          acc[m][v] -= (F1[v] - Qz[m][v]) * P::ih(Dl, 2);
+          if (v < L::IM0) mb += Qz[m][v], mt += F1[v];
+        }
+        const long long g = (long long)k * nx + (x0 + lx);
+        finish_cell<R, L, MICRO>(
+            a, Dl, ph, C, stage, dt, k, ys[m], acc[m], mb, mt,
+            [&](int v) { return S::PREFETCH ? s_yn[(m * NV + v) * NT + tid] : Yn[v * ncell + g]; },
+            yo);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) Yo[v * ncell + g] = yo[v];
+        if constexpr (RES) {
+#pragma unroll
+          for (int v = 0; v < NV; ++v) ys[m][v] = yo[v];
+        }
+        if (stage == 2)
+          rate_max = fmax(rate_max, cell_rate_r<R, L>(C, yo, P::er(Dl, k), P::ih(Dl, 0), R(0),
+                                                      P::ih(Dl, 2)));
+      }
+    if (stage == 2) {
+      double bm;
+      if constexpr (sizeof(R) == 4)
+        bm = double(block_max_f(rate_max, reinterpret_cast<float *>(s_red + 1)));
+      else
+        bm = block_max(rate_max, s_red + 1);
+      if (tid == 0)
+        atomicMax(RES ? D.rate_next : D.rate, (unsigned long long)__double_as_longlong(bm));
+    }
+    __syncthreads();
+  }
+}
+
 // The march along z (snap_march.cuh), for the tile shapes that ask for it.
 template <class R, class L, class T>
 struct MarchSmem;
@@ -1749,18 +2196,34 @@ __device__ __forceinline__ void run_stage(const StageArgs &a, int st, unsigned c
   if constexpr (T::MARCH) {
     static_assert(!VISC, "the march is built for inviscid layouts");
     march_tiles<R, L, T, MICRO, false>(a, st, smem);
-  } else {
-    R ys[Box<T, L::D3>::CPT][L::NV];
+  } else if constexpr (L::D3) {
+    R ys[Box<T, true>::CPT][L::NV];
     stage_tiles<R, L, VISC, T, MICRO>(a, st, smem, ys);
+  } else {
+    R ys[PlaneSmem<R, L, VISC, T>::M][L::NV];
+    plane_tiles<R, L, VISC, T, MICRO>(a, st, smem, ys);
   }
+}
+
+// Cells per thread whose state the resident step keeps in registers.
+template <class R, class L, bool VISC, class T>
+constexpr int kept_cells() {
+  if constexpr (T::MARCH)
+    return 1;
+  else if constexpr (L::D3)
+    return Box<T, true>::CPT;
+  else
+    return PlaneSmem<R, L, VISC, T>::M;
 }
 
 template <class R, class L, bool VISC, class T>
 constexpr size_t stage_smem() {
   if constexpr (T::MARCH)
     return MarchSmem<R, L, T>::total;
-  else
+  else if constexpr (L::D3)
     return StageSmem<R, L, VISC, T>::total;
+  else
+    return PlaneSmem<R, L, VISC, T>::total;
 }
 
 // One Runge-Kutta stage over all tiles of all domains.
@@ -1792,7 +2255,7 @@ template <class R, class L, bool VISC, class T, bool MICRO>
 __global__ void __launch_bounds__(T::NT, T::MINB) resident_step_kernel(const StageArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned int s_seq;
-  R ys[T::MARCH ? 1 : Box<T, L::D3>::CPT][L::NV];
+  R ys[kept_cells<R, L, VISC, T>()][L::NV];
   const int tile = blockIdx.x, tid = threadIdx.x;
   if (tid == 0) s_seq = ld_acquire_u32(&a.res->seq);
   __syncthreads();
@@ -1819,8 +2282,10 @@ __global__ void __launch_bounds__(T::NT, T::MINB) resident_step_kernel(const Sta
     // either ends with a CTA barrier
     if constexpr (T::MARCH)
       march_tiles<R, L, T, MICRO, true>(a, st, smem);
-    else
+    else if constexpr (L::D3)
       stage_tiles<R, L, VISC, T, MICRO, true>(a, st, smem, ys);
+    else
+      plane_tiles<R, L, VISC, T, MICRO, true>(a, st, smem, ys);
     if (st < 2 && tid == 0) {
       __threadfence();
       st_release_u32(a.tile_flags + tile, 3u * seq + unsigned(st) + 1u);
