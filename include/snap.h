@@ -252,7 +252,8 @@ int snap_use_graph(snap_ctx *ctx, int enable);
  * snap_info.n_tile_variants; the active one in snap_info.tile_variant). A new context starts
  * on the first shape, in the order built, whose tiles over all domains are at least the
  * device's SM count, else on the shape with the most tiles, so that a small grid still
- * spreads over every SM. In three dimensions (inviscid) the first shape is a march along z: tiles
+ * spreads over every SM. In the x-z plane a shape's height is an upper limit: the library takes
+ * fewer rows per tile where that spreads a small grid over more SMs (snap_info.tile). In three dimensions (inviscid) the first shape is a march along z: tiles
  * of 32 x 8 columns by a number of levels the library picks for the grid (snap_info.tile); it is
  * the default unless the grid is too small for it. Domains are re-tiled; results do not depend
  * on the shape. */

@@ -515,22 +515,49 @@ static long long count_tiles(const std::vector<DomDev> &doms, const int *tl, int
   return t;
 }
 
-// Levels per tile of a marching shape, and what a stage costs with them in units of one level of
-// one tile on one SM: the busiest SM walks n = ceil(tiles / SMs) tiles of cz + 3 levels' work
-// (three levels' conversions and two z reconstructions go into the start of a tile). A tile alone
-// on its SM takes about 1.4 times its share of a full SM (its barriers and loads are not hidden
-// by another tile). Against a fixed 16 levels: the radiative-convective column 128 x 96 x 128
-// (288 tiles of 22 levels, two per SM at once, instead of 384) 1.33 -> 1.08 ms per step, dry 190 x
-// 131 x 85 (408 tiles of 22 levels instead of 612 of 16) 0.65 -> 0.47 ms.
-static int march_levels(const std::vector<DomDev> &doms, const TileVariant &tv, int nsm,
-                        double *cost) {
+// Levels per tile of shape tv on the domains doms, and what a stage costs with them, where the
+// busiest SM works through n = ceil(tiles / SMs) tiles.
+//   March: in units of one level of one tile on one SM, n (cz + 3) (three levels' conversions and
+//     two z reconstructions go into the start of a tile). A tile alone on its SM takes about 1.4
+//     times its share of a full SM (its barriers and loads are not hidden by another tile). Against
+//     a fixed 16 levels: the radiative-convective column 128 x 96 x 128 (288 tiles of 22 levels,
+//     two per SM at once, instead of 384) 1.33 -> 1.08 ms per step, dry 190 x 131 x 85 (408 tiles of
+//     22 levels instead of 612 of 16) 0.65 -> 0.47 ms.
+//   x-z tiles: rows are dealt to the SM's four schedulers warp by warp, cz of them along x and
+//     cz + 2 along z, plus about a row's worth of conversions and barriers. Full tiles come
+//     first, the ragged top ones fill the SMs that a last round of full ones leaves idle. On a
+//     grid that fills the SMs this keeps the shape's full height; a small grid gets lower tiles
+//     on more SMs: 128 x 128 cells in FP64 (128 tiles of 4 rows instead of 40 of 14) 233 -> 95 us
+//     per step, the Bryan bubble 200 x 100 in FP64 864 -> 405 us, one moist bubble of 61 x 47 cells in
+//     FP32 29 -> 20 us.
+//   One-shot 3-D tiles: their own height.
+static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv, int nsm,
+                         double *cost) {
   int nzmax = 0, best = tv.tile[2];
-  for (const DomDev &D : doms) nzmax = D.nz > nzmax ? D.nz : nzmax;
   *cost = 1e300;
-  for (int cz = tv.tile[2]; cz >= 4; --cz) {
+  if (tv.levels == kFixedLevels) return best;
+  for (const DomDev &D : doms) nzmax = D.nz > nzmax ? D.nz : nzmax;
+  const bool march = tv.levels == kMarchLevels;
+  const auto quarter = [&](int rows) { return (rows * tv.tile[0] + 127) / 128; };
+  for (int cz = tv.tile[2]; cz >= (march ? 4 : 1); --cz) {
     if (cz >= 2 * nzmax) continue;
-    const long long n = (count_tiles(doms, tv.tile, cz) + nsm - 1) / nsm;
-    const double c = (cz + 3) * (n == 1 ? 1.4 : double(n));
+    double c;
+    if (march) {
+      const long long n = (count_tiles(doms, tv.tile, cz) + nsm - 1) / nsm;
+      c = (cz + 3) * (n == 1 ? 1.4 : double(n));
+    } else {
+      const auto work = [&](int rows) { return double(quarter(rows) + quarter(rows + 2) + 1); };
+      long long full = 0;
+      double ragged = 0.0;  // work of the top tiles
+      for (const DomDev &D : doms) {
+        const long long cols = (D.nx + tv.tile[0] - 1) / tv.tile[0];
+        full += cols * (D.nz / cz);
+        if (D.nz % cz) ragged += double(cols) * work(D.nz % cz);
+      }
+      const long long q = full / nsm, r = full % nsm;
+      const double idle = r ? double(nsm - r) * work(cz) : 0.0;
+      c = double(q + (r ? 1 : 0)) * work(cz) + (ragged > idle ? (ragged - idle) / nsm + 1.0 : 0.0);
+    }
     if (c < *cost) {
       *cost = c;
       best = cz;
@@ -542,12 +569,9 @@ static int march_levels(const std::vector<DomDev> &doms, const TileVariant &tv, 
 // Divides the domains into the tiles of shape tv, numbered from 0; prefix receives the first
 // tile of each domain and the total.
 static void tile_domains(std::vector<DomDev> &doms, const TileVariant &tv, int *prefix) {
-  int cz = tv.tile[2];
-  if (tv.march) {
-    double cost;
-    const int nsm = device_sms();
-    cz = march_levels(doms, tv, nsm > 0 ? nsm : 1, &cost);
-  }
+  double cost;
+  const int nsm = device_sms();
+  const int cz = choose_levels(doms, tv, nsm > 0 ? nsm : 1, &cost);
   prefix[0] = 0;
   for (size_t i = 0; i < doms.size(); ++i) {
     DomDev &D = doms[i];
@@ -575,16 +599,16 @@ static int default_variant(const snap_ctx *ctx) {
   long long best_tiles = -1;
   for (int v = 0; v < ctx->ks.nvariants; ++v) {
     const TileVariant &tv = ctx->ks.var[v];
-    if (tv.march) {
+    double cost;
+    const int cz = choose_levels(ctx->dom, tv, nsm, &cost);
+    if (tv.levels == kMarchLevels) {
       if (v + 1 == ctx->ks.nvariants) return v;
-      double cost;
-      march_levels(ctx->dom, tv, nsm, &cost);
       const int *tl = ctx->ks.var[v + 1].tile;
       const long long n = (count_tiles(ctx->dom, tl, tl[2]) + nsm - 1) / nsm;
       if (cost <= std::max(1.55 * n, 2.4)) return v;
       continue;
     }
-    const long long t = count_tiles(ctx->dom, tv.tile, tv.tile[2]);
+    const long long t = count_tiles(ctx->dom, tv.tile, cz);
     if (t >= nsm) return v;
     if (t > best_tiles) {
       best_tiles = t;

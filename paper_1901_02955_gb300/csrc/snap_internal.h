@@ -133,10 +133,13 @@ struct StageArgs {
 
 enum Flag : unsigned int { kFlagNonFinite = 1u, kFlagNoConv = 2u, kFlagTimeout = 4u };
 
+// Levels per tile (DomDev::cz): always tile[2], or chosen for the grid up to it.
+enum LevelChoice : int { kFixedLevels = 0, kMarchLevels = 1, kPlaneLevels = 2 };
+
 // One tile shape of a kernel family.
 struct TileVariant {
-  int tile[3];               // march: tile[2] is the most levels a tile may have
-  int march;                 // 1: walked level by level (snap_march.cuh)
+  int tile[3];               // tile[2]: the most levels a tile may have
+  int levels;                // how the levels per tile are chosen (LevelChoice)
   int threads;
   size_t smem_stage;
   cudaError_t (*stage)(const StageArgs &, int grid, cudaStream_t);

@@ -1909,8 +1909,9 @@ __device__ __forceinline__ void plane_tiles(const StageArgs &a, const int stage,
     const int lt = tile - D.tile_begin;
     int ix, iz;
     divide(lt, D.tx, D.tx_magic, iz, ix);
-    const int x0 = ix * TX, z0 = iz * TZ;
-    const int ex = min(TX, nx - x0), ez = min(TZ, nz - z0);
+    const int cz = D.cz;  // rows per tile, at most TZ
+    const int x0 = ix * TX, z0 = iz * cz;
+    const int ex = min(TX, nx - x0), ez = min(cz, nz - z0);
     const R *Ys = reinterpret_cast<const R *>(a.buf_s ? a.buf_s : D.buf[stage]);
     const R *Yn = reinterpret_cast<const R *>(a.buf_n ? a.buf_n : D.buf[0]);
     R *Yo = reinterpret_cast<R *>(a.buf_o ? a.buf_o : D.buf[stage == 0 ? 1 : (stage == 1 ? 2 : 0)]);
@@ -2527,7 +2528,7 @@ struct Variant {
     v.tile[0] = T::TX;
     v.tile[1] = T::TY;
     v.tile[2] = T::TZ;
-    v.march = T::MARCH;
+    v.levels = T::MARCH ? kMarchLevels : (L::D3 ? kFixedLevels : kPlaneLevels);
     v.threads = T::NT;
     v.smem_stage = kSmem;
     v.stage = &stage;
