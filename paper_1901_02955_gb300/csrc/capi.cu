@@ -517,9 +517,11 @@ static long long count_tiles(const std::vector<DomDev> &doms, const int *tl, int
 
 // Levels per tile of shape tv on the domains doms, and what a stage costs with them, where the
 // busiest SM works through n = ceil(tiles / SMs) tiles.
-//   March: in units of one level of one tile on one SM, n (cz + 3) (three levels' conversions and
-//     two z reconstructions go into the start of a tile). A tile alone on its SM takes about 1.4
-//     times its share of a full SM (its barriers and loads are not hidden by another tile). Against
+//   March: in units of one level of 256 columns on one SM, n (cz + 3) (three levels' conversions
+//     and two z reconstructions go into the start of a tile). A tile of 256 columns alone on its SM
+//     takes about 1.4 times its share of a full SM (its barriers and loads are not hidden by
+//     another tile), so a last round of fewer tiles than are resident costs up to 0.4 more; one of 512 costs 1.92 (many per SM: Jovian 256 x 256 x 128 at 8.04 against
+//     8.38 ms for two steps) to 2.1 of 256 (two per SM: 300 x 200 x 64, 4.74 against 4.21 ms). Against
 //     a fixed 16 levels: the radiative-convective column 128 x 96 x 128 (288 tiles of 22 levels,
 //     two per SM at once, instead of 384) 1.33 -> 1.08 ms per step, dry 190 x 131 x 85 (408 tiles of
 //     22 levels instead of 612 of 16) 0.65 -> 0.47 ms.
@@ -538,13 +540,17 @@ static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv,
   if (tv.levels == kFixedLevels) return best;
   for (const DomDev &D : doms) nzmax = D.nz > nzmax ? D.nz : nzmax;
   const bool march = tv.levels == kMarchLevels;
+  const int resident = march ? std::max(1, tv.max_resident_blocks() / nsm) : 1;
   const auto quarter = [&](int rows) { return (rows * tv.tile[0] + 127) / 128; };
   for (int cz = tv.tile[2]; cz >= (march ? 4 : 1); --cz) {
     if (cz >= 2 * nzmax) continue;
     double c;
     if (march) {
       const long long n = (count_tiles(doms, tv.tile, cz) + nsm - 1) / nsm;
-      c = (cz + 3) * (n == 1 ? 1.4 : double(n));
+      const int left = int(n % resident);  // tiles of the last round
+      c = (cz + 3) * (tv.tile[0] * tv.tile[1] == 512
+                          ? (n < 5 ? 2.1 : 1.92) * n
+                          : n + (left ? 0.4 * (resident - left) / std::max(1, resident - 1) : 0.0));
     } else {
       const auto work = [&](int rows) { return double(quarter(rows) + quarter(rows + 2) + 1); };
       long long full = 0;
@@ -587,35 +593,41 @@ static void tile_domains(std::vector<DomDev> &doms, const TileVariant &tv, int *
   }
 }
 
-// Default tile shape. A marching shape (first in its set) unless the grid is so small that the
-// one-shot tiles after it finish sooner: one such tile of 256 cells costs an SM 1.55 levels of a
+// Default tile shape. The cheaper marching shape (they come first in their set) unless the grid is
+// so small that the one-shot tiles after them finish sooner: one such tile of 256 cells costs an SM 1.55 levels of a
 // marching tile (Jovian 8.6 against 5.5 us, dry 4.3 against 2.8), and no less than 2.4 when the
 // SM has only one or two. Else the first shape (in the order built, the fastest on large grids)
 // whose tiles over all domains fill every SM at least once; else the one with the most tiles.
 static int default_variant(const snap_ctx *ctx) {
   const int nsm = device_sms();
   if (nsm <= 0) return 0;
-  int best = 0;
+  int best = 0, march = -1;
   long long best_tiles = -1;
+  double march_cost = 1e300;
   for (int v = 0; v < ctx->ks.nvariants; ++v) {
     const TileVariant &tv = ctx->ks.var[v];
     double cost;
     const int cz = choose_levels(ctx->dom, tv, nsm, &cost);
     if (tv.levels == kMarchLevels) {
-      if (v + 1 == ctx->ks.nvariants) return v;
-      const int *tl = ctx->ks.var[v + 1].tile;
-      const long long n = (count_tiles(ctx->dom, tl, tl[2]) + nsm - 1) / nsm;
-      if (cost <= std::max(1.55 * n, 2.4)) return v;
+      if (cost < march_cost) {
+        march_cost = cost;
+        march = v;
+      }
       continue;
     }
     const long long t = count_tiles(ctx->dom, tv.tile, cz);
+    if (march >= 0) {  // this is the first shape after the marching ones
+      const long long n = (t + nsm - 1) / nsm;
+      if (march_cost <= std::max(1.55 * n, 2.4)) return march;
+      march = -1;
+    }
     if (t >= nsm) return v;
     if (t > best_tiles) {
       best_tiles = t;
       best = v;
     }
   }
-  return best;
+  return march >= 0 ? march : best;
 }
 
 extern "C" int snap_init_grid(snap_ctx **out, const snap_grid_desc *d, int n_domains) {

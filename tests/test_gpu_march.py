@@ -67,14 +67,18 @@ def test_dry_march_equals_tiles_bitwise(n, dtype, walls):
 def test_moist_march_agrees_with_tiles(n, full):
     make = W.jovian_rce if full else W.jovian
     w = W.add_random_motion(make(nx=n[0], ny=n[1], nz=n[2], Lx=390.0 * n[0], Ly=390.0 * n[1]))
-    ref, _ = advance(w, "f32", 1, 0)
+    tiles = 1 if full else 2  # the one-shot shape follows the marching ones
+    ref, info = advance(w, "f32", tiles, 0)
+    assert info["tile"] == (8, 8, 4)
     scale = np.abs(ref).reshape(w.nv, -1).max(axis=1)
-    for mode in (0, 1, 2):
-        out, _ = advance(w, "f32", 0, mode)
-        if out is None:
-            continue
-        d = np.abs(out - ref).reshape(w.nv, -1).max(axis=1)
-        assert np.all(d <= 1e-6 * np.maximum(scale, 1e-30)), (mode, d / scale)
+    for v in range(tiles):
+        for mode in (0, 1, 2):
+            out, info = advance(w, "f32", v, mode)
+            assert info["tile"][0] == 32
+            if out is None:
+                continue
+            d = np.abs(out - ref).reshape(w.nv, -1).max(axis=1)
+            assert np.all(d <= 1e-6 * np.maximum(scale, 1e-30)), (v, mode, d / scale)
 
 
 def test_march_over_linked_slabs_equals_the_whole_domain():
