@@ -206,11 +206,13 @@ int snap_saturation_adjust(snap_ctx *ctx, int domain);
 /* Forward run recorded for the adjoint: advances the domain by nsteps steps like snap_step,
  * keeping the final state, the time step of every step and
  *   ckpt_every >= 1: a checkpoint of the state every ckpt_every steps; the adjoint recomputes
- *     each segment from its checkpoint. Allocates nsteps/ckpt_every + 2 state copies and a
- *     segment of 3 x ckpt_every states (the input of each of the three stages of a step);
+ *     each segment from its checkpoint, but for the last one, whose stage inputs the forward
+ *     run keeps. Allocates nsteps/ckpt_every + 2 state copies and one or two segments of 3 x
+ *     ckpt_every states (the input of each of the three stages of a step);
  *   ckpt_every == 0: the input of every stage of every step (3 x nsteps + 1 state copies);
  *     the adjoint recomputes nothing.
- * Also allocates four adjoint vectors and the per-face work arrays of the adjoint. The
+ * Also allocates four adjoint vectors and the per-face work arrays of the adjoint. The memory of
+ * the last record serves the next one where it is large enough; snap_free returns it. The
  * adjoint is built for a single inviscid domain, dry (x-z or 3-D) or with one vapour and two
  * condensates in the x-z plane, with free-slip or periodic sides and no fixed bottom
  * temperature; SNAP_ENOTSUP for any other context. */

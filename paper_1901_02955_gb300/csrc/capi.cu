@@ -181,6 +181,9 @@ struct snap_ctx {
   void *ckpt = nullptr;       // checkpoints every ckpt_every steps, then the final state
   void *segbuf = nullptr;     // states of one segment, or of two (see snap_step_adjoint)
   int nsegbuf = 1;
+  size_t ckpt_bytes = 0, segbuf_bytes = 0;  // sizes of the two, and room of dt_hist
+  int dt_hist_room = 0;
+  int seg_held = -1;          // segment whose stage inputs segbuf holds since snap_record (-1: none)
   cudaStream_t rec_stream = nullptr;  // recomputation of the next segment
   cudaEvent_t ev_rec[2] = {nullptr, nullptr}, ev_free[2] = {nullptr, nullptr};
   double *dt_hist = nullptr;  // device copy of the recorded time steps
@@ -1374,25 +1377,44 @@ extern "C" int snap_record(snap_ctx *ctx, int nsteps, int ckpt_every, double dt_
   // store_all: the final state only; else every ckpt_every-th state and the final one
   const int nck = store_all ? 1 : (nsteps + ckpt_every - 1) / ckpt_every + 1;
   const int nseg_states = store_all ? nsteps : ckpt_every;
+  const int nseg = store_all ? 1 : (nsteps + ckpt_every - 1) / ckpt_every;
   ctx->rec_steps = 0;
-  cudaFree(ctx->ckpt);
-  cudaFree(ctx->segbuf);
-  ctx->ckpt = ctx->segbuf = nullptr;
-  CK(cudaMalloc(&ctx->ckpt, sb * nck));
+  ctx->seg_held = -1;
+  // The buffers of the last record serve again where they are large enough (and not more than
+  // four times too large): a record allocated and freed 126 MB per call (256 x 256 cells, FP32, 40
+  // steps), 0.3 ms of a 5.6 ms gradient.
+  auto fits = [](size_t have, size_t need) { return have >= need && have / 4 <= need; };
+  if (!fits(ctx->ckpt_bytes, sb * nck)) {
+    cudaFree(ctx->ckpt);
+    ctx->ckpt = nullptr;
+    ctx->ckpt_bytes = 0;
+    CK(cudaMalloc(&ctx->ckpt, sb * nck));
+    ctx->ckpt_bytes = sb * nck;
+  }
   // per step: the inputs of its three stages (Y^n and the results of stages 0 and 1); with
   // more than one segment, room for two segments, so that the adjoint recomputes the next
   // segment while it transposes the current one (one segment's room if two do not fit)
-  ctx->nsegbuf = 1;
-  if (!store_all && nsteps > ckpt_every) {
-    if (cudaMalloc(&ctx->segbuf, sb * 3 * nseg_states * 2) == cudaSuccess)
-      ctx->nsegbuf = 2;
-    else
+  const size_t segb = sb * 3 * nseg_states;
+  ctx->nsegbuf = nseg > 1 ? 2 : 1;
+  if (!fits(ctx->segbuf_bytes, segb * ctx->nsegbuf)) {
+    cudaFree(ctx->segbuf);
+    ctx->segbuf = nullptr;
+    ctx->segbuf_bytes = 0;
+    if (cudaMalloc(&ctx->segbuf, segb * ctx->nsegbuf) != cudaSuccess) {
       cudaGetLastError();
+      ctx->segbuf = nullptr;
+      ctx->nsegbuf = 1;
+      CK(cudaMalloc(&ctx->segbuf, segb));
+    }
+    ctx->segbuf_bytes = segb * ctx->nsegbuf;
   }
-  if (!ctx->segbuf) CK(cudaMalloc(&ctx->segbuf, sb * 3 * nseg_states));
-  cudaFree(ctx->dt_hist);
-  ctx->dt_hist = nullptr;
-  CK(cudaMalloc(&ctx->dt_hist, sizeof(double) * nsteps));
+  if (ctx->dt_hist_room < nsteps) {
+    cudaFree(ctx->dt_hist);
+    ctx->dt_hist = nullptr;
+    ctx->dt_hist_room = 0;
+    CK(cudaMalloc(&ctx->dt_hist, sizeof(double) * nsteps));
+    ctx->dt_hist_room = nsteps;
+  }
   if (!ctx->lam) CK(cudaMalloc(&ctx->lam, sb * 4));
   if (!ctx->gface) {
     const DomDev &D = ctx->dom[0];
@@ -1424,27 +1446,30 @@ extern "C" int snap_record(snap_ctx *ctx, int nsteps, int ckpt_every, double dt_
   ctx->ckpt_every = ckpt_every;
   const int keep = ctx->use_graph;
   const StageArgs base = args_of(ctx, 0);
-  if (store_all) {
-    int rc = set_dt_fixed(ctx, dt_fixed);
-    if (rc) return rc;
-  }
+  // The steps whose stage inputs go straight into the record: all of them, or with checkpoints
+  // those of the last segment, which the adjoint transposes first (it would otherwise be
+  // recomputed, with nothing to overlap it).
+  const int last0 = store_all ? 0 : (nseg - 1) * ckpt_every;
+  char *last_buf = (char *)ctx->segbuf + (ctx->nsegbuf == 2 ? segb * ((nseg - 1) & 1) : 0);
   for (int n = 0; n < nsteps; ++n) {
-    if (store_all) {
-      // three launches per step writing straight into the record: the inputs of the stages
-      // of step n are slots 3n, 3n+1, 3n+2; stage 2 writes the next step's slot (the
-      // context's state after the last step)
-      const DomDev &D = ctx->dom[0];
-      char *slot = (char *)ctx->segbuf + sb * 3 * n;
-      if (n == 0) CK(cudaMemcpyAsync(slot, D.buf[0], sb, cudaMemcpyDeviceToDevice, ctx->stream));
+    const DomDev &D = ctx->dom[0];
+    if (!store_all && n % ckpt_every == 0)
+      CK(cudaMemcpyAsync((char *)ctx->ckpt + sb * (n / ckpt_every), D.buf[0], sb,
+                         cudaMemcpyDeviceToDevice, ctx->stream));
+    if (n >= last0) {
+      // three launches per step: the inputs of the stages of step n are slots 3m, 3m+1, 3m+2,
+      // m = n - last0; stage 2 writes the next step's slot (the context's state after the last
+      // step)
+      int rc = SNAP_OK;
+      if (n == last0 && (rc = set_dt_fixed(ctx, dt_fixed))) return rc;
+      char *slot = last_buf + sb * 3 * (n - last0);
+      if (n == last0) CK(cudaMemcpyAsync(slot, D.buf[0], sb, cudaMemcpyDeviceToDevice, ctx->stream));
       void *next = n + 1 < nsteps ? (void *)(slot + 3 * sb) : D.buf[0];
-      int rc = plain_stage(ctx, base, 0, -1.0, slot, slot, slot + sb);
+      rc = plain_stage(ctx, base, 0, -1.0, slot, slot, slot + sb);
       if (!rc) rc = plain_stage(ctx, base, 1, -1.0, slot + sb, slot, slot + 2 * sb);
       if (!rc) rc = plain_stage(ctx, base, 2, -1.0, slot + 2 * sb, slot, next);
       if (rc) return rc;
     } else {
-      if (n % ckpt_every == 0)
-        CK(cudaMemcpyAsync((char *)ctx->ckpt + sb * (n / ckpt_every), ctx->dom[0].buf[0], sb,
-                           cudaMemcpyDeviceToDevice, ctx->stream));
       int rc = snap_step_async(ctx, 1, dt_fixed);
       if (rc) return rc;
     }
@@ -1458,6 +1483,7 @@ extern "C" int snap_record(snap_ctx *ctx, int nsteps, int ckpt_every, double dt_
   CK(cudaStreamSynchronize(ctx->stream));
   ctx->use_graph = keep;
   ctx->rec_steps = nsteps;
+  if (!store_all) ctx->seg_held = nseg - 1;
   return snap_check(ctx, nullptr);
 }
 
@@ -1570,7 +1596,7 @@ extern "C" int snap_step_adjoint(snap_ctx *ctx, int nsteps, const void *lambda_f
     // the recomputation stream starts after the work queued so far (the adjoint's input)
     CK(cudaEventRecord(ctx->ev_free[1], ctx->stream));
     CK(cudaStreamWaitEvent(ctx->rec_stream, ctx->ev_free[1], 0));
-    rc = recompute(nseg - 1, ctx->rec_stream);
+    if (ctx->seg_held != nseg - 1) rc = recompute(nseg - 1, ctx->rec_stream);
     if (!rc) CK(cudaEventRecord(ctx->ev_rec[(nseg - 1) & 1], ctx->rec_stream));
   }
   for (int seg = nseg - 1; seg >= 0 && rc == SNAP_OK; --seg) {
@@ -1585,9 +1611,11 @@ extern "C" int snap_step_adjoint(snap_ctx *ctx, int nsteps, const void *lambda_f
         CK(cudaEventRecord(ctx->ev_rec[b ^ 1], ctx->rec_stream));
       }
       CK(cudaStreamWaitEvent(ctx->stream, ctx->ev_rec[b], 0));
-    } else if (!store_all) {
+    } else if (!store_all && ctx->seg_held != seg) {
       if ((rc = recompute(seg, ctx->stream))) break;
     }
+    // the buffers go to other segments from here on (one segment alone stays in its buffer)
+    if (nseg > 1) ctx->seg_held = -1;
     char *buf = store_all ? (char *)ctx->segbuf : segment_buffer(seg);
     for (int s = n1 - 1; s >= n0 && rc == SNAP_OK; --s) {
       const double dt = ctx->rec_dt[s];
