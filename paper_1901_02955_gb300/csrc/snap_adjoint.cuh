@@ -15,7 +15,7 @@
 //     G[d][face][s][v] (v padded to a 16-byte vector, so that each slot moves as one access);
 //   FP64 instead: adj_prim_kernel (primitives of every cell once), adj_weno_kernel (every
 //     five-cell window once: both face states it yields and their gradients, sharing the
-//     smoothness indicators) and adj_face_w_kernel (LMARS transposed from the stored states,
+//     smoothness indicators, in pairs of floats) and adj_face_w_kernel (LMARS transposed from the stored states,
 //     the same G) -- about a third less work on the slow FP64 pipe;
 //   adj_cell_kernel: one thread per cell gathers the contributions of every face whose
 //     stencil holds the cell (or a ghost image of it), transposes the primitive map and the
@@ -282,6 +282,105 @@ __device__ __forceinline__ void weno5_pair_grad(const R q[5], R eps, R &QL, R &Q
   // do not change), so each gradient sums to one: the centre entries follow from the others
   gL[2] = R(1) - ((gL[0] + gL[1]) + (gL[3] + gL[4]));
   gR[2] = R(1) - ((gR[0] + gR[1]) + (gR[3] + gR[4]));
+}
+
+// An FP64 number as a pair of floats and back by integer instructions (a conversion instruction to
+// or from FP64 holds the FP64 pipe as long as an addition): the top 24 bits of the mantissa, and the
+// remaining 29 rounded to 24. ok is cleared outside 2^-73 .. 2^127 (zero is fine).
+__device__ __forceinline__ Df split64(double x, bool &ok) {
+  const int hi = __double2hiint(x), lo = __double2loint(x), e = (hi >> 20) & 0x7ff;
+  const int sign = hi & 0x80000000;
+  if (e < 950 || e > 1149) {
+    ok = ok && x == 0.0;
+    return {0.0f, 0.0f};
+  }
+  // the exponent fields differ by 896, which mod 256 flips the float field's top bit
+  const int h = sign | ((__funnelshift_l(lo, hi, 3) ^ 0x40000000) & 0x7fffffff);
+  const float l = __int2float_rn(lo & 0x1fffffff) * __int_as_float((e - 948) << 23);
+  return {__int_as_float(h), __int_as_float(__float_as_int(l) ^ sign)};
+}
+__device__ __forceinline__ double widen(float f) {  // a subnormal f counts as zero
+  const int b = __float_as_int(f);
+  const int hi = (b & 0x80000000) | (((b & 0x7fffffff) >> 3) + (896 << 20));
+  return (b & 0x7f800000) ? __hiloint2double(hi, b << 29) : 0.0;
+}
+__device__ __forceinline__ double join64(Df x) { return widen(x.h) + widen(x.l); }
+__device__ __forceinline__ Df times2(Df a) { return {2.0f * a.h, 2.0f * a.l}; }
+__device__ __forceinline__ Df neg(Df a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ Df recip(Df a) {
+  const float r = Ar<float>::rcp(a.h);
+  return quick2(r, __fmul_rn(r, __fmaf_rn(-r, a.l, __fmaf_rn(-r, a.h, 1.0f))));
+}
+
+// weno5_pair_grad in pairs of floats. Only the four neighbour differences, the centre value and the
+// results are FP64; the indicators, weights and their derivatives carry about 46 bits (the FP64
+// form's shared reciprocal is good to 1e-12). With w = q0 - q1, u = q2 - q1, v = q3 - q2,
+// z = q3 - q4, s0 = u + w, s1 = v - u, s2 = v + z, r0 = 3 u + w, r1 = u + v, r2 = 3 v + z the
+// indicators are s_k^2 + 3/13 r_k^2 and the candidates' offsets from q2
+//   left state s0/12 + r0/4, s1/12 + r1/4, -s2/12 + r2/4; right state the same with -r_k/4.
+// The gradient runs back from the weighted sum of the offsets d_k through the weights w_k
+// (-2 w_k / e_k sum_j w_j (d_k - d_j): a difference from the sum itself would cancel where one
+// weight is near one, as beside a jump), the indicators e_k and the differences. Against the
+// textbook formula in extended precision, 65,536 windows each: gradients to 3e-16 .. 4e-14 rms of
+// their largest entry on random, smooth and jump windows (the FP64 form: 2e-13 .. 8e-12), states to 2e-15 of
+// the window's largest value or better (5e-14). False (nothing written) where a difference or an indicator leaves the range in
+// which the floats' exponents hold every product; the caller then takes the FP64 form.
+//
+// The window kernel is bound by the FP64 pipe in the FP64 form (145 operations per field and
+// window at 68 to 80 cycles a warp); here 30 are left beside about 1250 FP32 instructions: 155 -> 74 us a launch (dry, 256 x 256 cells).
+__device__ __forceinline__ bool weno5_pair_grad_pairs(const double q[5], double eps, double &QL,
+                                                      double &QR, double gL[5], double gR[5]) {
+  bool ok = true;
+  const Df u = split64(q[2] - q[1], ok), v = split64(q[3] - q[2], ok);
+  const Df w = split64(q[0] - q[1], ok), z = split64(q[3] - q[4], ok);
+  if (!ok) return false;
+  constexpr Df k3 = {0.23076923191547394f, -1.1462431004360951e-09f};  // 3/13
+  constexpr Df k12 = {0.0833333358168602f, -2.4835269396561444e-09f};  // 1/12
+  const Df s0 = u + w, s1 = v - u, s2 = v + z;
+  const Df r0 = times2(u) + s0, r1 = u + v, r2 = times2(v) + s2;
+  const Df t0 = k3 * r0, t1 = k3 * r1, t2 = k3 * r2;
+  const float ef = float(eps * (12.0 / 13.0));
+  const Df ep = {ef, float(eps * (12.0 / 13.0) - double(ef))};
+  const Df e0 = ep + (s0 * s0 + t0 * r0), e1 = ep + (s1 * s1 + t1 * r1),
+           e2 = ep + (s2 * s2 + t2 * r2);
+  const float elo = fminf(e0.h, fminf(e1.h, e2.h)), ehi = fmaxf(e0.h, fmaxf(e1.h, e2.h));
+  if (!(elo > 1e-15f && ehi < 1e15f)) return false;
+  const Df i0 = recip(e0), i1 = recip(e1), i2 = recip(e2);
+  const Df g0 = i0 * i0, g1 = (i1 * i1) * 6.0f, g2 = i2 * i2;  // g1 with its linear weight
+  const Df g03 = g0 * 3.0f, g23 = g2 * 3.0f;
+  const Df iL = recip((g0 + g1) + g23), iR = recip((g03 + g1) + g2);
+  const Df n0 = times2(neg(i0)), n1 = times2(neg(i1)), n2 = times2(neg(i2));  // -2 / e_k
+  const Df a0 = s0 * k12, a1 = s1 * k12, a2 = neg(s2 * k12);
+  // one state: weights w_k, sg the sign of its r terms; returns the offset from q2
+  const auto side = [&](Df w0, Df w1, Df w2, float sg, double *g) {
+    const float sr = 0.25f * sg;
+    const Df d0 = a0 + Df{sr * r0.h, sr * r0.l}, d1 = a1 + Df{sr * r1.h, sr * r1.l},
+             d2 = a2 + Df{sr * r2.h, sr * r2.l};
+    const Df d01 = d0 - d1, d02 = d0 - d2, d12 = d1 - d2;
+    const Df x0 = (w1 * d01 + w2 * d02) * (w0 * n0);
+    const Df x1 = (w2 * d12 - w0 * d01) * (w1 * n1);
+    const Df x2 = neg(w0 * d02 + w1 * d12) * (w2 * n2);
+    const auto lin = [&](Df y) { return Df{sr * y.h, sr * y.l}; };
+    const Df S0 = times2(x0 * s0) + w0 * k12, S1 = times2(x1 * s1) + w1 * k12,
+             S2 = times2(x2 * s2) - w2 * k12;
+    const Df R0 = times2(x0 * t0) + lin(w0), R1 = times2(x1 * t1) + lin(w1),
+             R2 = times2(x2 * t2) + lin(w2);
+    const double ub = join64(((S0 - S1) + R0 * 3.0f) + R1);
+    const double vb = join64(((S1 + S2) + R2 * 3.0f) + R1);
+    const double wb = join64(S0 + R0), zb = join64(S2 + R2);
+    g[0] = wb;
+    g[1] = -(ub + wb);
+    g[2] = (1.0 + ub) - vb;
+    g[3] = vb + zb;
+    g[4] = -zb;
+    return join64((w0 * d0 + w1 * d1) + w2 * d2);
+  };
+  double h[5];
+  QL = q[2] + side(g0 * iL, g1 * iL, g23 * iL, 1.0f, gL);
+  QR = q[2] + side(g03 * iR, g1 * iR, g2 * iR, -1.0f, h);
+#pragma unroll
+  for (int t = 0; t < 5; ++t) gR[4 - t] = h[t];
+  return true;
 }
 
 // Transpose of mix_factors<>: adds the adjoint of (num, den) to the tracer entries of Xb.
@@ -641,7 +740,12 @@ __device__ __forceinline__ void adj_window(const AdjArgs &a, const DomDev &D, lo
       const R x = X[v * ncell + cs[t]];
       q[t] = (v == MN && fl[t]) ? -x : x;
     }
-    weno5_pair_grad<R>(q, weps, QL, QR, gL, gR);
+    if constexpr (sizeof(R) == 8) {
+      if (!weno5_pair_grad_pairs(q, weps, QL, QR, gL, gR))
+        weno5_pair_grad<R>(q, weps, QL, QR, gL, gR);
+    } else {
+      weno5_pair_grad<R>(q, weps, QL, QR, gL, gR);
+    }
     W[v * nc + e] = QL;
     W[(NV + v) * nc + e] = QR;
 #pragma unroll
