@@ -1383,30 +1383,38 @@ extern "C" int snap_record(snap_ctx *ctx, int nsteps, int ckpt_every, double dt_
   // The buffers of the last record serve again where they are large enough (and not more than
   // four times too large): a record allocated and freed 126 MB per call (256 x 256 cells, FP32, 40
   // steps), 0.3 ms of a 5.6 ms gradient.
-  auto fits = [](size_t have, size_t need) { return have >= need && have / 4 <= need; };
-  if (!fits(ctx->ckpt_bytes, sb * nck)) {
-    cudaFree(ctx->ckpt);
-    ctx->ckpt = nullptr;
-    ctx->ckpt_bytes = 0;
-    CK(cudaMalloc(&ctx->ckpt, sb * nck));
-    ctx->ckpt_bytes = sb * nck;
-  }
+  auto take = [](void *&p, size_t &have, size_t need) {
+    if (have >= need && have / 4 <= need) return true;
+    cudaFree(p);
+    p = nullptr;
+    have = 0;
+    if (cudaMalloc(&p, need) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+      return false;
+    }
+    have = need;
+    return true;
+  };
   // per step: the inputs of its three stages (Y^n and the results of stages 0 and 1); with
   // more than one segment, room for two segments, so that the adjoint recomputes the next
-  // segment while it transposes the current one (one segment's room if two do not fit)
+  // segment while it transposes the current one (one segment's room if two do not fit). What
+  // does not fit beside the last record's buffers is tried again without them.
   const size_t segb = sb * 3 * nseg_states;
   ctx->nsegbuf = nseg > 1 ? 2 : 1;
-  if (!fits(ctx->segbuf_bytes, segb * ctx->nsegbuf)) {
+  auto take_both = [&] {
+    return take(ctx->ckpt, ctx->ckpt_bytes, sb * nck) &&
+           take(ctx->segbuf, ctx->segbuf_bytes, segb * ctx->nsegbuf);
+  };
+  if (!take_both()) {
+    cudaFree(ctx->ckpt);
     cudaFree(ctx->segbuf);
-    ctx->segbuf = nullptr;
-    ctx->segbuf_bytes = 0;
-    if (cudaMalloc(&ctx->segbuf, segb * ctx->nsegbuf) != cudaSuccess) {
-      cudaGetLastError();
-      ctx->segbuf = nullptr;
+    ctx->ckpt = ctx->segbuf = nullptr;
+    ctx->ckpt_bytes = ctx->segbuf_bytes = 0;
+    if (!take_both()) {
       ctx->nsegbuf = 1;
-      CK(cudaMalloc(&ctx->segbuf, segb));
+      if (!take_both()) return cuda_fail(ctx, cudaErrorMemoryAllocation, "snap_record");
     }
-    ctx->segbuf_bytes = segb * ctx->nsegbuf;
   }
   if (ctx->dt_hist_room < nsteps) {
     cudaFree(ctx->dt_hist);
