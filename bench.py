@@ -133,7 +133,8 @@ def kernel_sources_md5(kern="kern_dry2d.cu"):
     committed ncu traffic figure."""
     h = hashlib.md5()
     csrc = os.path.join(ROOT, "paper_1901_02955_gb300", "csrc")
-    for f in ("snap_stage.cuh", "snap_internal.h", kern):
+    march = ("snap_march.cuh",) if "3d" in kern else ()
+    for f in ("snap_stage.cuh", "snap_internal.h", *march, kern):
         h.update(open(os.path.join(csrc, f), "rb").read())
     return h.hexdigest()
 
