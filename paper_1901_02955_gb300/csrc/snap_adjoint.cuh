@@ -327,7 +327,8 @@ __device__ __forceinline__ Df recip(Df a) {
 // which the floats' exponents hold every product; the caller then takes the FP64 form.
 //
 // The window kernel is bound by the FP64 pipe in the FP64 form (145 operations per field and
-// window at 68 to 80 cycles a warp); here 30 are left beside about 1250 FP32 instructions: 155 -> 74 us a launch (dry, 256 x 256 cells).
+// window at 68 to 80 cycles a warp); here 30 are left beside about 1250 FP32 instructions: 155 -> 60 us
+// a launch (dry, 256 x 256 cells; 76 where the caller's loop over the fields was unrolled).
 __device__ __forceinline__ bool weno5_pair_grad_pairs(const double q[5], double eps, double &QL,
                                                       double &QR, double gL[5], double gR[5]) {
   bool ok = true;
@@ -732,7 +733,10 @@ __device__ __forceinline__ void adj_window(const AdjArgs &a, const DomDev &D, lo
     cs[t] = ((long long)ck * ny + cj) * nx + ci;
   }
   const R weps = acst<R>(a).weno_eps;
-#pragma unroll
+  // a loop, not a copy per field and direction of these 1300 instructions and the fallback's: the copies
+  // left the instruction cache (ncu: 6.6 cycles of every issue waited for instructions). Gradient of 10
+  // FP64 steps on 256 x 256 cells 9.00 -> 8.64 ms.
+#pragma unroll 1
   for (int v = 0; v < NV; ++v) {
     R q[5], QL, QR, gL[5], gR[5];
 #pragma unroll
