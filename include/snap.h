@@ -406,10 +406,18 @@ int snap_probe_fma(int dtype, double *tflops, void *stream);
  * dtype, laid out [n][5]; out [n][2] receives the kernels' WENO5 states of Sec. 4.2 (Eq. weno5
  * with the Jiang-Shu indicators and the given eps): the left state at face c+1/2 and the
  * right state at face c-1/2. packed = 1 (SNAP_F32, n even) runs windows 2p and 2p+1 through
- * the packed two-variable form the FP32 kernels use for pairs of variables. */
+ * the packed two-variable form the FP32 kernels use for pairs of variables.
+ *
+ * snap_check_weno_grad: the FP64 adjoint's window operation on n windows of five doubles: out
+ * [n][13] receives the left state at face c+1/2, the right state at face c-1/2, the left state's
+ * derivatives by the window's values in order, the right state's in reversed order (by e first),
+ * and 1 where the window was taken in pairs of floats, 0 where in FP64. fp64 = 1: every window in
+ * FP64. */
 int snap_check_rcp64(const double *x, double *y, long long n, void *stream);
 int snap_check_weno(int dtype, int packed, const void *win, void *out, long long n, double eps,
                     void *stream);
+int snap_check_weno_grad(const double *win, double *out, long long n, double eps, int fp64,
+                         void *stream);
 
 void snap_free(snap_ctx *ctx);
 const char *snap_last_error(const snap_ctx *ctx);

@@ -32,7 +32,7 @@ EXPORTS = ["snap_init_grid", "snap_set_state", "snap_get_state", "snap_step", "s
            "snap_set_barrier_test", "snap_link_halo", "snap_halo_buffer", "snap_halo_pack",
            "snap_set_class_tile_variant", "snap_get_class_info",
            "snap_get_info", "snap_buffer_pointer", "snap_budget_noalloc", "snap_theta_e",
-           "snap_probe_fma", "snap_check_rcp64", "snap_check_weno",
+           "snap_probe_fma", "snap_check_rcp64", "snap_check_weno", "snap_check_weno_grad",
            "snap_free", "snap_last_error", "snap_status_string"]
 
 
@@ -125,6 +125,7 @@ def load(path: Optional[str] = None) -> C.CDLL:
     lib.snap_probe_fma.argtypes = [C.c_int, C.POINTER(C.c_double), P]
     lib.snap_check_rcp64.argtypes = [P, P, C.c_longlong, P]
     lib.snap_check_weno.argtypes = [C.c_int, C.c_int, P, P, C.c_longlong, C.c_double, P]
+    lib.snap_check_weno_grad.argtypes = [P, P, C.c_longlong, C.c_double, C.c_int, P]
     lib.snap_budget_noalloc.argtypes = [P, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,
                                         C.c_int, C.c_double, C.c_double, C.c_double,
                                         C.c_double, P, P]
@@ -450,6 +451,14 @@ def check_weno(dtype, packed, win_ptr, out_ptr, n, eps, stream=None):
                                 n, eps, stream)
     if rc:
         raise SnapError(rc, "snap_check_weno failed")
+
+
+def check_weno_grad(win_ptr, out_ptr, n, eps, fp64=False, stream=None):
+    """Device pointers: states and gradients of n five-value windows as the FP64 adjoint forms
+    them (see snap_check_weno_grad)."""
+    rc = load().snap_check_weno_grad(win_ptr, out_ptr, n, eps, int(fp64), stream)
+    if rc:
+        raise SnapError(rc, "snap_check_weno_grad failed")
 
 
 def probe_fma(dtype="f32", stream=None):

@@ -4,12 +4,12 @@
 // issue, so their roofline is quoted against the FP32 fused multiply-add rate; this measures
 // that rate (and the FP64 one) on the device and clocks at hand, next to the nominal figure.
 // It also holds the arithmetic self-checks: the stage kernels' FP64 reciprocal and WENO5
-// reconstruction run on caller-given arguments, for tests against IEEE division and the
-// textbook formula.
+// reconstruction and the FP64 adjoint's window gradients run on caller-given arguments, for tests
+// against IEEE division and the textbook formula.
 #include <cuda_runtime.h>
 
 #include "../../include/snap.h"
-#include "snap_stage.cuh"
+#include "snap_adjoint.cuh"
 
 namespace {
 
@@ -105,6 +105,25 @@ __global__ void weno_packed_kernel(const float *win, float *out, long long npair
   }
 }
 
+// per window: left state, right state, their gradients (weno5_pair_grad's order) and 1 where the pairs
+// of floats took the window
+__global__ void weno_grad_kernel(const double *win, double *out, long long n, double eps, int fp64) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+       i += (long long)gridDim.x * blockDim.x) {
+    const double *q = win + 5 * i;
+    double *o = out + 13 * i, QL, QR, gL[5], gR[5];
+    const bool pairs = !fp64 && snap::weno5_pair_grad_pairs(q, eps, QL, QR, gL, gR);
+    if (!pairs) snap::weno5_pair_grad<double>(q, eps, QL, QR, gL, gR);
+    o[0] = QL;
+    o[1] = QR;
+    for (int t = 0; t < 5; ++t) {
+      o[2 + t] = gL[t];
+      o[7 + t] = gR[t];
+    }
+    o[12] = pairs ? 1.0 : 0.0;
+  }
+}
+
 int grid_for(long long n) {
   const long long g = (n + kThreads - 1) / kThreads;
   return int(g < 4096 ? (g > 0 ? g : 1) : 4096);
@@ -135,6 +154,14 @@ extern "C" int snap_check_weno(int dtype, int packed, const void *win, void *out
   else
     weno_kernel<double><<<grid_for(n), kThreads, 0, s>>>((const double *)win, (double *)out, n,
                                                          eps);
+  return cudaGetLastError() == cudaSuccess ? SNAP_OK : SNAP_ECUDA;
+}
+
+extern "C" int snap_check_weno_grad(const double *win, double *out, long long n, double eps,
+                                    int fp64, void *stream) {
+  if (n < 0 || (n > 0 && (!win || !out))) return SNAP_EINVAL;
+  if (n == 0) return SNAP_OK;
+  weno_grad_kernel<<<grid_for(n), kThreads, 0, (cudaStream_t)stream>>>(win, out, n, eps, fp64);
   return cudaGetLastError() == cudaSuccess ? SNAP_OK : SNAP_ECUDA;
 }
 

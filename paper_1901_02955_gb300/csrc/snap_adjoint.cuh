@@ -286,11 +286,12 @@ __device__ __forceinline__ void weno5_pair_grad(const R q[5], R eps, R &QL, R &Q
 
 // An FP64 number as a pair of floats and back by integer instructions (a conversion instruction to
 // or from FP64 holds the FP64 pipe as long as an addition): the top 24 bits of the mantissa, and the
-// remaining 29 rounded to 24. ok is cleared outside 2^-73 .. 2^127 (zero is fine).
+// remaining 29 rounded to 24. ok is cleared outside 2^-73 .. 2^60 (zero is fine): the float holds more,
+// but the square of a value from 2^64 on leaves it.
 __device__ __forceinline__ Df split64(double x, bool &ok) {
   const int hi = __double2hiint(x), lo = __double2loint(x), e = (hi >> 20) & 0x7ff;
   const int sign = hi & 0x80000000;
-  if (e < 950 || e > 1149) {
+  if (e < 950 || e > 1082) {
     ok = ok && x == 0.0;
     return {0.0f, 0.0f};
   }
@@ -324,7 +325,9 @@ __device__ __forceinline__ Df recip(Df a) {
 // textbook formula in extended precision, 65,536 windows each: gradients to 3e-16 .. 4e-14 rms of
 // their largest entry on random, smooth and jump windows (the FP64 form: 2e-13 .. 8e-12), states to 2e-15 of
 // the window's largest value or better (5e-14). False (nothing written) where a difference or an indicator leaves the range in
-// which the floats' exponents hold every product; the caller then takes the FP64 form.
+// which the floats' exponents hold every product; the caller then takes the FP64 form. Every indicator
+// is tested by itself: a minimum or maximum over them would drop a NaN, which is what an overflow in
+// the pairs ends in (infinity minus infinity).
 //
 // The window kernel is bound by the FP64 pipe in the FP64 form (145 operations per field and
 // window at 68 to 80 cycles a warp); here 30 are left beside about 1250 FP32 instructions: 155 -> 60 us
@@ -344,8 +347,8 @@ __device__ __forceinline__ bool weno5_pair_grad_pairs(const double q[5], double 
   const Df ep = {ef, float(eps * (12.0 / 13.0) - double(ef))};
   const Df e0 = ep + (s0 * s0 + t0 * r0), e1 = ep + (s1 * s1 + t1 * r1),
            e2 = ep + (s2 * s2 + t2 * r2);
-  const float elo = fminf(e0.h, fminf(e1.h, e2.h)), ehi = fmaxf(e0.h, fmaxf(e1.h, e2.h));
-  if (!(elo > 1e-15f && ehi < 1e15f)) return false;
+  const auto inside = [](Df e) { return e.h > 1e-15f && e.h < 1e15f; };
+  if (!(inside(e0) && inside(e1) && inside(e2))) return false;
   const Df i0 = recip(e0), i1 = recip(e1), i2 = recip(e2);
   const Df g0 = i0 * i0, g1 = (i1 * i1) * 6.0f, g2 = i2 * i2;  // g1 with its linear weight
   const Df g03 = g0 * 3.0f, g23 = g2 * 3.0f;
