@@ -284,15 +284,20 @@ __device__ __forceinline__ void weno5_pair_grad(const R q[5], R eps, R &QL, R &Q
   gR[2] = R(1) - ((gR[0] + gR[1]) + (gR[3] + gR[4]));
 }
 
+__device__ __forceinline__ bool below_pairs(double x) {  // |x| < 2^-73
+  return (__double2hiint(x) & 0x7ff00000) < (950 << 20);
+}
 // An FP64 number as a pair of floats and back by integer instructions (a conversion instruction to
 // or from FP64 holds the FP64 pipe as long as an addition): the top 24 bits of the mantissa, and the
-// remaining 29 rounded to 24. ok is cleared outside 2^-73 .. 2^60 (zero is fine): the float holds more,
-// but the square of a value from 2^64 on leaves it.
-__device__ __forceinline__ Df split64(double x, bool &ok) {
+// remaining 29 rounded to 24. ok is cleared from 2^60 on: the float holds more, but the square of a value
+// from 2^64 on leaves it. Below 2^-73 (the low part would lose bits) the pair is zero, and tiny is set
+// unless x is.
+__device__ __forceinline__ Df split64(double x, bool &ok, bool &tiny) {
   const int hi = __double2hiint(x), lo = __double2loint(x), e = (hi >> 20) & 0x7ff;
   const int sign = hi & 0x80000000;
-  if (e < 950 || e > 1082) {
-    ok = ok && x == 0.0;
+  if (e > 1082) ok = false;
+  if (e < 950) {
+    tiny = tiny || (unsigned(hi) << 1 | unsigned(lo)) != 0u;
     return {0.0f, 0.0f};
   }
   // the exponent fields differ by 896, which mod 256 flips the float field's top bit
@@ -323,20 +328,26 @@ __device__ __forceinline__ Df recip(Df a) {
 // (-2 w_k / e_k sum_j w_j (d_k - d_j): a difference from the sum itself would cancel where one
 // weight is near one, as beside a jump), the indicators e_k and the differences. Against the
 // textbook formula in extended precision, 65,536 windows each: gradients to 3e-16 .. 4e-14 rms of
-// their largest entry on random, smooth and jump windows (the FP64 form: 2e-13 .. 8e-12), states to 2e-15 of
-// the window's largest value or better (5e-14). False (nothing written) where a difference or an indicator leaves the range in
-// which the floats' exponents hold every product; the caller then takes the FP64 form. Every indicator
-// is tested by itself: a minimum or maximum over them would drop a NaN, which is what an overflow in
-// the pairs ends in (infinity minus infinity).
+// their largest entry on random, smooth and jump windows (the FP64 form: 2e-13 .. 8e-12), states to
+// 2e-15 of the window's largest value or better (5e-14).
+//
+// False (nothing written) where a difference or an indicator is too large, or an indicator too small,
+// for the floats' exponents to hold every product; the caller then takes the FP64 form. Every
+// indicator is tested by itself: a minimum or maximum over them would drop a NaN, which is what an
+// overflow in the pairs ends in (infinity minus infinity). A difference below 2^-73 is left out of the
+// indicators and gradients (it is at most 3e-15 of the square root of an indicator) and enters the
+// states in FP64: ahead of what moves a field at rest has little else, and with the FP64 form for such
+// windows their warps ran both (per adjoint step from rest, 64 x 64 cells 184 against 145 us, 256 x 256
+// 490 against 398 us; in the FP64 form alone 171 and 673 us).
 //
 // The window kernel is bound by the FP64 pipe in the FP64 form (145 operations per field and
 // window at 68 to 80 cycles a warp); here 30 are left beside about 1250 FP32 instructions: 155 -> 60 us
 // a launch (dry, 256 x 256 cells; 76 where the caller's loop over the fields was unrolled).
 __device__ __forceinline__ bool weno5_pair_grad_pairs(const double q[5], double eps, double &QL,
                                                       double &QR, double gL[5], double gR[5]) {
-  bool ok = true;
-  const Df u = split64(q[2] - q[1], ok), v = split64(q[3] - q[2], ok);
-  const Df w = split64(q[0] - q[1], ok), z = split64(q[3] - q[4], ok);
+  bool ok = true, tiny = false;
+  const Df u = split64(q[2] - q[1], ok, tiny), v = split64(q[3] - q[2], ok, tiny);
+  const Df w = split64(q[0] - q[1], ok, tiny), z = split64(q[3] - q[4], ok, tiny);
   if (!ok) return false;
   constexpr Df k3 = {0.23076923191547394f, -1.1462431004360951e-09f};  // 3/13
   constexpr Df k12 = {0.0833333358168602f, -2.4835269396561444e-09f};  // 1/12
@@ -377,7 +388,18 @@ __device__ __forceinline__ bool weno5_pair_grad_pairs(const double q[5], double 
     g[2] = (1.0 + ub) - vb;
     g[3] = vb + zb;
     g[4] = -zb;
-    return join64((w0 * d0 + w1 * d1) + w2 * d2);
+    double off = join64((w0 * d0 + w1 * d1) + w2 * d2);
+    if (tiny) {
+      const auto rest = [](double x) { return below_pairs(x) ? x : 0.0; };
+      const double du = rest(q[2] - q[1]), dv = rest(q[3] - q[2]);
+      const double dw = rest(q[0] - q[1]), dz = rest(q[3] - q[4]);
+      const double W0 = join64(w0), W1 = join64(w1), W2 = join64(w2);
+      off += sg > 0.0f ? (1.0 / 6.0) * (W0 * (5.0 * du + 2.0 * dw) + W1 * (du + 2.0 * dv) +
+                                        W2 * (4.0 * dv + dz))
+                       : (-1.0 / 6.0) * (W0 * (4.0 * du + dw) + W1 * (2.0 * du + dv) +
+                                         W2 * (5.0 * dv + 2.0 * dz));
+    }
+    return off;
   };
   double h[5];
   QL = q[2] + side(g0 * iL, g1 * iL, g23 * iL, 1.0f, gL);

@@ -115,6 +115,24 @@ def test_every_scale(torch, eps):
     assert same(out[~pairs], ref[~pairs]) and not ref[:, 12].any()
 
 
+def test_windows_near_rest_stay_in_pairs(torch):
+    """Differences below 2^-73 = 1.1e-22 (a field at rest far from what moves) leave the indicators
+    and gradients as they are, 1e-22 against sqrt(eps) = 1e-3, but not the states: the same bounds,
+    relative to the window's own largest value, for windows of 1e-23 down to the subnormal numbers
+    and for windows that mix them with zeros and with larger values at every position."""
+    rs = np.random.default_rng(24)
+    m, X = 300, []
+    for q in (-21, -22, -23, -25, -40, -150, -290, -310):
+        Y = rs.normal(size=(m, 5)) * 10.0 ** q
+        X += [Y, np.where(rs.random((m, 5)) < 0.4, 0.0, Y),
+              np.where(rs.random((m, 5)) < 0.3, rs.normal(size=(m, 5)), Y),
+              np.where(rs.random((m, 5)) < 0.3, 1e-18 * rs.normal(size=(m, 5)), Y)]
+    X = np.concatenate(X)
+    out = run(torch, X, 1e-6)
+    assert np.all(out[:, 12] == 1.0)
+    check_pairs(X, out, 1e-6)
+
+
 @pytest.mark.parametrize("jump", [1e8, 1.9e19, 1e20, 1e30])
 @pytest.mark.parametrize("step", [False, True])
 def test_jumps_beyond_the_range(torch, jump, step):
