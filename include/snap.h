@@ -264,7 +264,9 @@ int snap_set_tile_variant(snap_ctx *ctx, int variant);
 /* Launch mode of a step. 0 (default): three launches per step, one per stage. 1: one
  * persistent cooperative launch whose CTAs (all co-resident) walk the tile queue of every
  * domain and meet at a grid barrier between the three stages. 2: the resident step, for grids
- * whose tiles are all co-resident at once (SNAP_ENOTSUP otherwise, or with SNAP_HALO sides):
+ * whose tiles are all co-resident at once (SNAP_ENOTSUP otherwise, or with SNAP_HALO sides;
+ * where the tile height picked for three launches gives more tiles than that, the domains are
+ * re-tiled for the resident step, and back when the mode is left):
  * one cooperative launch with one tile per CTA; each CTA keeps its tile's state on chip
  * through the three stages and, between stages, waits only for the tiles its ghost cells
  * come from (a flag per tile) instead of for the whole grid. Every device-side wait of modes

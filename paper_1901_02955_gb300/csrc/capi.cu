@@ -159,6 +159,7 @@ struct snap_ctx {
   int *dep_begin = nullptr, *dep_list = nullptr;
   unsigned long long *rate_next_dev = nullptr;
   int res_ready = 0, res_tv = -1;
+  int tile_cap = 0;  // most tiles the current tiling was allowed (0: any number)
   // size classes (domains of identical nx, ny, nz) and their own tile shapes: with per_class
   // set (three-launch mode only), a stage is one launch per class on parallel streams, each
   // over the class's own tile table (cls_dom, uploaded to cls_doms_dev / cls_prefix_dev)
@@ -536,8 +537,10 @@ static long long count_tiles(const std::vector<DomDev> &doms, const int *tl, int
 //     per step, the Bryan bubble 200 x 100 in FP64 864 -> 405 us, one moist bubble of 61 x 47 cells in
 //     FP32 29 -> 20 us.
 //   One-shot 3-D tiles: their own height.
+//
+// cap > 0: no more than cap tiles, if a height allows it (the resident step's co-resident CTAs).
 static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv, int nsm,
-                         double *cost) {
+                         double *cost, int cap = 0) {
   int nzmax = 0, best = tv.tile[2];
   *cost = 1e300;
   if (tv.levels == kFixedLevels) return best;
@@ -547,6 +550,7 @@ static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv,
   const auto quarter = [&](int rows) { return (rows * tv.tile[0] + 127) / 128; };
   for (int cz = tv.tile[2]; cz >= (march ? 4 : 1); --cz) {
     if (cz >= 2 * nzmax) continue;
+    if (cap > 0 && count_tiles(doms, tv.tile, cz) > cap) continue;
     double c;
     if (march) {
       const long long n = (count_tiles(doms, tv.tile, cz) + nsm - 1) / nsm;
@@ -577,10 +581,11 @@ static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv,
 
 // Divides the domains into the tiles of shape tv, numbered from 0; prefix receives the first
 // tile of each domain and the total.
-static void tile_domains(std::vector<DomDev> &doms, const TileVariant &tv, int *prefix) {
+static void tile_domains(std::vector<DomDev> &doms, const TileVariant &tv, int *prefix,
+                         int cap = 0) {
   double cost;
   const int nsm = device_sms();
-  const int cz = choose_levels(doms, tv, nsm > 0 ? nsm : 1, &cost);
+  const int cz = choose_levels(doms, tv, nsm > 0 ? nsm : 1, &cost, cap);
   prefix[0] = 0;
   for (size_t i = 0; i < doms.size(); ++i) {
     DomDev &D = doms[i];
@@ -858,9 +863,11 @@ extern "C" int snap_init_grid(snap_ctx **out, const snap_grid_desc *d, int n_dom
   return SNAP_OK;
 }
 
-// Rebuild the tile tables of every domain for tile variant v and upload them.
-static int apply_variant(snap_ctx *ctx, int v) {
-  tile_domains(ctx->dom, ctx->ks.var[v], ctx->prefix.data());
+// Rebuild the tile tables of every domain for tile variant v (at most cap tiles, 0: any number) and
+// upload them.
+static int retile(snap_ctx *ctx, int v, int cap) {
+  tile_domains(ctx->dom, ctx->ks.var[v], ctx->prefix.data(), cap);
+  ctx->tile_cap = cap;
   ctx->ntiles = ctx->prefix[ctx->ndom];
   ctx->grid = ctx->ntiles;
   const int mrb = ctx->ks.var[v].max_resident_blocks();
@@ -868,8 +875,6 @@ static int apply_variant(snap_ctx *ctx, int v) {
   ctx->grid_persistent = mrb < ctx->ntiles ? mrb : ctx->ntiles;
   ctx->tv = v;
   ctx->res_ready = 0;
-  for (int &t : ctx->cls_tv) t = v;
-  ctx->per_class = 0;
   CK(cudaMemcpyAsync(ctx->doms_dev, ctx->dom.data(), sizeof(DomDev) * ctx->ndom,
                      cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemcpyAsync(ctx->prefix_dev, ctx->prefix.data(), sizeof(int) * (ctx->ndom + 1),
@@ -880,6 +885,13 @@ static int apply_variant(snap_ctx *ctx, int v) {
     ctx->graph = nullptr;
   }
   return SNAP_OK;
+}
+
+// Every domain, and every size class, on tile variant v.
+static int apply_variant(snap_ctx *ctx, int v) {
+  for (int &t : ctx->cls_tv) t = v;
+  ctx->per_class = 0;
+  return retile(ctx, v, 0);
 }
 
 static cudaStream_t pick(snap_ctx *ctx, void *stream) {
@@ -1046,17 +1058,22 @@ static int ghost_source(int p, int n, bool periodic) {
   return p < 0 ? -1 - p : 2 * n - 1 - p;
 }
 
-// Whether the resident step can run the current tiling: every tile co-resident, and no slab
-// boundary (its ghost cells come from another domain's tiles).
+// Whether the resident step can run the current tile shape: every tile co-resident at some height
+// (the height picked for three launches may give more tiles than that), and no slab boundary (its
+// ghost cells come from another domain's tiles).
 static bool resident_possible(snap_ctx *ctx, std::string *why) {
   for (int i = 0; i < ctx->ndom; ++i)
     if (ctx->dom[i].bc[0] == kBcHalo || ctx->dom[i].bc[1] == kBcHalo) {
       if (why) *why = "the resident step does not take slab boundaries (SNAP_HALO)";
       return false;
     }
-  const int mrt = ctx->ks.var[ctx->tv].max_resident_tiles();
-  if (mrt <= 0 || ctx->ntiles > mrt) {
-    if (why) *why = "the resident step needs every tile co-resident (" + std::to_string(ctx->ntiles) +
+  const TileVariant &tv = ctx->ks.var[ctx->tv];
+  const int mrt = tv.max_resident_tiles(), nsm = device_sms();
+  double cost;
+  const int cz = choose_levels(ctx->dom, tv, nsm > 0 ? nsm : 1, &cost, mrt);
+  const long long least = std::min<long long>(ctx->ntiles, count_tiles(ctx->dom, tv.tile, cz));
+  if (mrt <= 0 || least > mrt) {
+    if (why) *why = "the resident step needs every tile co-resident (" + std::to_string(least) +
                     " tiles, " + std::to_string(mrt) + " co-resident CTAs for this tile shape)";
     return false;
   }
@@ -1071,6 +1088,11 @@ static bool resident_possible(snap_ctx *ctx, std::string *why) {
 static int build_resident(snap_ctx *ctx) {
   std::string why;
   if (!resident_possible(ctx, &why)) return fail(ctx, SNAP_ENOTSUP, "snap_use_persistent: " + why);
+  const int mrt = ctx->ks.var[ctx->tv].max_resident_tiles();
+  if (ctx->ntiles > mrt) {
+    const int rc = retile(ctx, ctx->tv, mrt);
+    if (rc) return rc;
+  }
   const int *shape = ctx->ks.var[ctx->tv].tile;
   const int nt = ctx->ntiles;
   std::vector<std::vector<int>> dep(nt);
@@ -1734,6 +1756,9 @@ extern "C" int snap_use_persistent(snap_ctx *ctx, int enable) {
     return fail(ctx, SNAP_ECUDA, "snap_use_persistent: no co-resident CTA for the step kernel");
   if (enable == 2) {
     const int rc = build_resident(ctx);
+    if (rc) return rc;
+  } else if (ctx->tile_cap) {  // the tiling was the resident step's
+    const int rc = retile(ctx, ctx->tv, 0);
     if (rc) return rc;
   }
   ctx->persistent = enable;

@@ -137,17 +137,18 @@ __device__ __forceinline__ const CstT<double> &cst<double>(const StageArgs &a) {
 
 // Tile shape: TX x TY x TZ owned cells per CTA of NT threads (TY = 1 in the x-z plane).
 // MINB: CTAs per SM the kernel is compiled for (second __launch_bounds__ argument), which caps
-// its registers; 0 leaves the register count to the compiler.
-template <int TX_, int TY_, int TZ_, int NT_ = 256, int MINB_ = 0>
+// its registers; 0 leaves the register count to the compiler. RESB: the same for the resident step,
+// which takes no grid of more tiles than are co-resident.
+template <int TX_, int TY_, int TZ_, int NT_ = 256, int MINB_ = 0, int RESB_ = MINB_>
 struct TileT {
-  static constexpr int TX = TX_, TY = TY_, TZ = TZ_, NT = NT_, MINB = MINB_;
+  static constexpr int TX = TX_, TY = TY_, TZ = TZ_, NT = NT_, MINB = MINB_, RESB = RESB_;
   static constexpr bool MARCH = false;
 };
 // A tile of TX x TY columns of at most TZ levels (DomDev::cz of them) walked level by level, one
 // thread per column (snap_march.cuh).
 template <int TX_, int TY_, int TZ_, int MINB_ = 0>
 struct MarchT {
-  static constexpr int TX = TX_, TY = TY_, TZ = TZ_, NT = TX_ * TY_, MINB = MINB_;
+  static constexpr int TX = TX_, TY = TY_, TZ = TZ_, NT = TX_ * TY_, MINB = MINB_, RESB = MINB_;
   static constexpr bool MARCH = true;
 };
 
@@ -2280,7 +2281,7 @@ __global__ void __launch_bounds__(T::NT, T::MINB) step_kernel(const StageArgs a)
 // instead of a grid barrier or a new launch. Waits are bounded like the grid barrier's. The
 // last CTA to finish moves each domain's next CFL rate into place and advances seq.
 template <class R, class L, bool VISC, class T, bool MICRO>
-__global__ void __launch_bounds__(T::NT, T::MINB) resident_step_kernel(const StageArgs a) {
+__global__ void __launch_bounds__(T::NT, T::RESB) resident_step_kernel(const StageArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned int s_seq;
   R ys[kept_cells<R, L, VISC, T>()][L::NV];
