@@ -264,14 +264,13 @@ int snap_set_tile_variant(snap_ctx *ctx, int variant);
 /* Launch mode of a step. 0 (default): three launches per step, one per stage. 1: one
  * persistent cooperative launch whose CTAs (all co-resident) walk the tile queue of every
  * domain and meet at a grid barrier between the three stages. 2: the resident step, for grids
- * whose tiles are all co-resident at once (SNAP_ENOTSUP otherwise, or with SNAP_HALO sides;
- * where the tile height picked for three launches gives more tiles than that, the domains are
- * re-tiled for the resident step, and back when the mode is left):
- * one cooperative launch with one tile per CTA; each CTA keeps its tile's state on chip
- * through the three stages and, between stages, waits only for the tiles its ghost cells
- * come from (a flag per tile) instead of for the whole grid. Every device-side wait of modes
- * 1 and 2 is bounded (about 2 s) and reports SNAP_ETIMEOUT instead of hanging. Results are
- * the same in every mode. */
+ * whose tiles are all co-resident at once at the shape's full height (SNAP_ENOTSUP otherwise, or
+ * with SNAP_HALO sides): one cooperative launch with one tile per CTA; each CTA keeps its
+ * tile's state on chip through the three stages and, between stages, waits only for the tiles
+ * its ghost cells come from (a flag per tile) instead of for the whole grid. Every device-side wait of modes
+ * 1 and 2 is bounded (about 2 s) and reports SNAP_ETIMEOUT instead of hanging. Tile heights are
+ * picked for the mode (the domains are re-tiled when it changes). Results are the same in every
+ * mode. */
 int snap_use_persistent(snap_ctx *ctx, int enable);
 
 /* Test aid for the persistent step's grid barrier (the paper has no counterpart): each wait

@@ -8,6 +8,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <functional>
 #include <new>
 #include <string>
 #include <vector>
@@ -159,7 +160,7 @@ struct snap_ctx {
   int *dep_begin = nullptr, *dep_list = nullptr;
   unsigned long long *rate_next_dev = nullptr;
   int res_ready = 0, res_tv = -1;
-  int tile_cap = 0;  // most tiles the current tiling was allowed (0: any number)
+  int tile_mode = 0;  // launch mode the current tiling was made for
   // size classes (domains of identical nx, ny, nz) and their own tile shapes: with per_class
   // set (three-launch mode only), a stage is one launch per class on parallel streams, each
   // over the class's own tile table (cls_dom, uploaded to cls_doms_dev / cls_prefix_dev)
@@ -536,40 +537,79 @@ static long long count_tiles(const std::vector<DomDev> &doms, const int *tl, int
 //     on more SMs: 128 x 128 cells in FP64 (128 tiles of 4 rows instead of 40 of 14) 233 -> 95 us
 //     per step, the Bryan bubble 200 x 100 in FP64 864 -> 405 us, one moist bubble of 61 x 47 cells in
 //     FP32 29 -> 20 us.
+//     The top tiles' work spreads evenly over the SMs while every tile is co-resident, and about so
+//     over many rounds of several tiles per SM at once. Between one and two rounds, and where an SM
+//     holds one tile, a tile beyond the round waits for another to end and counts whole. Spread
+//     evenly there too, a few tiles spilt into another round: 446 x 108 moist FP64 (154 tiles of 10
+//     rows on 152 SMs; whole: 126 of 12) 668 -> 406 us per step, 768 x 256 dry FP32 (312 of 10 on 304
+//     places; 264 of 12) 35 -> 29 us, 628 x 229 moist FP32 (460 of 10 on 456; 400 of 12) 52 -> 41 us;
+//     at full height 535, 37 and 47 us with the kernels of before the lower tiles.
 //   One-shot 3-D tiles: their own height.
-//
-// cap > 0: no more than cap tiles, if a height allows it (the resident step's co-resident CTAs).
+// mode: the launch mode the tiling is for (snap_use_persistent). even: spread the top tiles' work
+// evenly whatever their number.
+//   2, the resident step: one tile per SM where that is possible, else as many as are co-resident.
 static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv, int nsm,
-                         double *cost, int cap = 0) {
+                         double *cost, int mode = 0, bool even = false) {
   int nzmax = 0, best = tv.tile[2];
   *cost = 1e300;
   if (tv.levels == kFixedLevels) return best;
   for (const DomDev &D : doms) nzmax = D.nz > nzmax ? D.nz : nzmax;
   const bool march = tv.levels == kMarchLevels;
-  const int resident = march ? std::max(1, tv.max_resident_blocks() / nsm) : 1;
+  const int resident = std::max(1, tv.max_resident_blocks() / nsm);
+  long long cap = 0;  // most tiles (0: any number)
+  if (mode == 2) {
+    cap = std::max(0, tv.max_resident_tiles());
+    if (count_tiles(doms, tv.tile, tv.tile[2]) <= nsm) cap = std::min<long long>(cap, nsm);
+  }
   const auto quarter = [&](int rows) { return (rows * tv.tile[0] + 127) / 128; };
+  const auto work = [&](int rows) { return quarter(rows) + quarter(rows + 2) + 1; };
   for (int cz = tv.tile[2]; cz >= (march ? 4 : 1); --cz) {
     if (cz >= 2 * nzmax) continue;
-    if (cap > 0 && count_tiles(doms, tv.tile, cz) > cap) continue;
+    const long long tiles = count_tiles(doms, tv.tile, cz);
+    if (cap > 0 && tiles > cap) continue;
     double c;
     if (march) {
-      const long long n = (count_tiles(doms, tv.tile, cz) + nsm - 1) / nsm;
+      const long long n = (tiles + nsm - 1) / nsm;
       const int left = int(n % resident);  // tiles of the last round
       c = (cz + 3) * (tv.tile[0] * tv.tile[1] == 512
                           ? (n < 5 ? 2.1 : 1.92) * n
                           : n + (left ? 0.4 * (resident - left) / std::max(1, resident - 1) : 0.0));
     } else {
-      const auto work = [&](int rows) { return double(quarter(rows) + quarter(rows + 2) + 1); };
       long long full = 0;
-      double ragged = 0.0;  // work of the top tiles
+      std::vector<long long> top(cz, 0);  // ragged top tiles by their rows
       for (const DomDev &D : doms) {
         const long long cols = (D.nx + tv.tile[0] - 1) / tv.tile[0];
         full += cols * (D.nz / cz);
-        if (D.nz % cz) ragged += double(cols) * work(D.nz % cz);
+        if (D.nz % cz) top[D.nz % cz] += cols;
       }
       const long long q = full / nsm, r = full % nsm;
+      double ragged = 0.0;  // work of the top tiles
+      for (int rows = 1; rows < cz; ++rows) ragged += double(top[rows]) * work(rows);
       const double idle = r ? double(nsm - r) * work(cz) : 0.0;
       c = double(q + (r ? 1 : 0)) * work(cz) + (ragged > idle ? (ragged - idle) / nsm + 1.0 : 0.0);
+      const long long slots = (long long)resident * nsm;
+      const double share = c;
+      if (!even && tiles > slots && (resident == 1 || tiles < 2 * slots)) {
+        c = 0.0;
+        if (mode == 1) {  // the CTAs take the tiles in turn: the first has one of every round
+          c += double((tiles + slots - 1) / slots) * resident * work(cz);
+        } else {  // higher top tiles first, each to the SM with the least work so far
+          std::vector<long long> load(nsm, q * work(cz));
+          for (int i = 0; i < int(r); ++i) load[i] += work(cz);
+          const auto later = std::greater<long long>();
+          std::make_heap(load.begin(), load.end(), later);
+          for (int rows = cz - 1; rows > 0; --rows) {
+            c += double(top[rows] / nsm) * work(rows);
+            for (long long i = top[rows] % nsm; i > 0; --i) {
+              std::pop_heap(load.begin(), load.end(), later);
+              load.back() += work(rows);
+              std::push_heap(load.begin(), load.end(), later);
+            }
+          }
+          c += double(*std::max_element(load.begin(), load.end()));
+        }
+      }
+      c += 1e-3 * share;  // decides between equals
     }
     if (c < *cost) {
       *cost = c;
@@ -582,10 +622,10 @@ static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv,
 // Divides the domains into the tiles of shape tv, numbered from 0; prefix receives the first
 // tile of each domain and the total.
 static void tile_domains(std::vector<DomDev> &doms, const TileVariant &tv, int *prefix,
-                         int cap = 0) {
+                         int mode = 0) {
   double cost;
   const int nsm = device_sms();
-  const int cz = choose_levels(doms, tv, nsm > 0 ? nsm : 1, &cost, cap);
+  const int cz = choose_levels(doms, tv, nsm > 0 ? nsm : 1, &cost, mode);
   prefix[0] = 0;
   for (size_t i = 0; i < doms.size(); ++i) {
     DomDev &D = doms[i];
@@ -615,7 +655,7 @@ static int default_variant(const snap_ctx *ctx) {
   for (int v = 0; v < ctx->ks.nvariants; ++v) {
     const TileVariant &tv = ctx->ks.var[v];
     double cost;
-    const int cz = choose_levels(ctx->dom, tv, nsm, &cost);
+    const int cz = choose_levels(ctx->dom, tv, nsm, &cost, 0, true);
     if (tv.levels == kMarchLevels) {
       if (cost < march_cost) {
         march_cost = cost;
@@ -863,11 +903,10 @@ extern "C" int snap_init_grid(snap_ctx **out, const snap_grid_desc *d, int n_dom
   return SNAP_OK;
 }
 
-// Rebuild the tile tables of every domain for tile variant v (at most cap tiles, 0: any number) and
-// upload them.
-static int retile(snap_ctx *ctx, int v, int cap) {
-  tile_domains(ctx->dom, ctx->ks.var[v], ctx->prefix.data(), cap);
-  ctx->tile_cap = cap;
+// Rebuild the tile tables of every domain for tile variant v in a launch mode and upload them.
+static int retile(snap_ctx *ctx, int v, int mode) {
+  tile_domains(ctx->dom, ctx->ks.var[v], ctx->prefix.data(), mode);
+  ctx->tile_mode = mode;
   ctx->ntiles = ctx->prefix[ctx->ndom];
   ctx->grid = ctx->ntiles;
   const int mrb = ctx->ks.var[v].max_resident_blocks();
@@ -891,7 +930,7 @@ static int retile(snap_ctx *ctx, int v, int cap) {
 static int apply_variant(snap_ctx *ctx, int v) {
   for (int &t : ctx->cls_tv) t = v;
   ctx->per_class = 0;
-  return retile(ctx, v, 0);
+  return retile(ctx, v, ctx->persistent);
 }
 
 static cudaStream_t pick(snap_ctx *ctx, void *stream) {
@@ -1070,10 +1109,10 @@ static bool resident_possible(snap_ctx *ctx, std::string *why) {
   const TileVariant &tv = ctx->ks.var[ctx->tv];
   const int mrt = tv.max_resident_tiles(), nsm = device_sms();
   double cost;
-  const int cz = choose_levels(ctx->dom, tv, nsm > 0 ? nsm : 1, &cost, mrt);
-  const long long least = std::min<long long>(ctx->ntiles, count_tiles(ctx->dom, tv.tile, cz));
-  if (mrt <= 0 || least > mrt) {
-    if (why) *why = "the resident step needs every tile co-resident (" + std::to_string(least) +
+  const int cz = choose_levels(ctx->dom, tv, nsm > 0 ? nsm : 1, &cost, 2);
+  const long long tiles = count_tiles(ctx->dom, tv.tile, cz);
+  if (mrt <= 0 || tiles > mrt) {
+    if (why) *why = "the resident step needs every tile co-resident (" + std::to_string(tiles) +
                     " tiles, " + std::to_string(mrt) + " co-resident CTAs for this tile shape)";
     return false;
   }
@@ -1088,9 +1127,8 @@ static bool resident_possible(snap_ctx *ctx, std::string *why) {
 static int build_resident(snap_ctx *ctx) {
   std::string why;
   if (!resident_possible(ctx, &why)) return fail(ctx, SNAP_ENOTSUP, "snap_use_persistent: " + why);
-  const int mrt = ctx->ks.var[ctx->tv].max_resident_tiles();
-  if (ctx->ntiles > mrt) {
-    const int rc = retile(ctx, ctx->tv, mrt);
+  if (ctx->tile_mode != 2) {
+    const int rc = retile(ctx, ctx->tv, 2);
     if (rc) return rc;
   }
   const int *shape = ctx->ks.var[ctx->tv].tile;
@@ -1757,8 +1795,8 @@ extern "C" int snap_use_persistent(snap_ctx *ctx, int enable) {
   if (enable == 2) {
     const int rc = build_resident(ctx);
     if (rc) return rc;
-  } else if (ctx->tile_cap) {  // the tiling was the resident step's
-    const int rc = retile(ctx, ctx->tv, 0);
+  } else if (ctx->tile_mode != enable) {
+    const int rc = retile(ctx, ctx->tv, enable);
     if (rc) return rc;
   }
   ctx->persistent = enable;
@@ -1798,11 +1836,13 @@ extern "C" int snap_autotune(snap_ctx *ctx, int steps, double *best_ms, int *cho
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   for (int v = 0; v < ctx->ks.nvariants && rc == SNAP_OK; ++v) {
+    ctx->persistent = 0;
     rc = apply_variant(ctx, v);
     for (int p = 0; p < 3 && rc == SNAP_OK; ++p) {
       if (p == 1 && ctx->grid_persistent <= 0) continue;
       if (p == 2 && !resident_possible(ctx, nullptr)) continue;
       ctx->persistent = p;
+      if (p && (rc = retile(ctx, v, p))) break;
       rc = snap_step_async(ctx, 1, 0.0);  // warm-up
       if (rc) break;
       CK(cudaEventRecord(e0, ctx->stream));
@@ -1881,11 +1921,10 @@ extern "C" int snap_autotune(snap_ctx *ctx, int steps, double *best_ms, int *cho
   cudaFree(save);
   ctx->use_graph = keep_graph;
   if (rc) return rc;
+  ctx->persistent = use_classes ? 0 : best_p;
   rc = apply_variant(ctx, best_v);
   if (rc) return rc;
-  ctx->persistent = best_p;
   if (use_classes) {
-    ctx->persistent = 0;
     ctx->cls_tv = cls_best;
     ctx->per_class = 1;
     if ((rc = build_class_tables(ctx))) return rc;

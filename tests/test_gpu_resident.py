@@ -2,7 +2,8 @@
 also where the height picked for three launches gives more tiles than that (a little more than one
 wave), and the moist FP64 layout with two tiles per SM. It equals three launches there (bitwise, with
 the saturation adjustment to 1e-6 of each field's largest value as in the other launch-mode tests),
-and the tiling for three launches is back when the mode is left."""
+and the tiling for three launches is back when the mode is left. In the other modes the heights do not
+spill a few tiles into another round."""
 import numpy as np
 import pytest
 
@@ -100,3 +101,26 @@ def test_autotune_tries_the_resident_step_where_it_fits():
     ctx.step(2)
     assert np.array_equal(ctx.get_state(), want)
     ctx.close()
+
+
+@pytest.mark.parametrize("make,dtype,nx,nz,nu,mode", [
+    (moist, "f64", 446, 108, 0.0, 0), (moist, "f32", 486, 344, 0.0, 0),
+    (moist, "f32", 628, 229, 0.0, 0), (dry, "f32", 768, 256, 0.0, 0),
+    (dry, "f32", 1039, 179, 75.0, 0), (dry, "f64", 544, 160, 0.0, 0),
+    (dry, "f64", 544, 160, 0.0, 1), (dry, "f64", 282, 427, 75.0, 1),
+    (moist, "f64", 346, 162, 0.0, 1)])
+def test_heights_do_not_spill_a_few_tiles_into_another_round(make, dtype, nx, nz, nu, mode):
+    """The heights keep such grids within the co-resident tiles, or well into the next round: a few
+    tiles more than are co-resident cost a whole round (446 x 108 moist FP64: 154 tiles on 152
+    places, 1.6 times the step of 126)."""
+    import torch
+    from paper_1901_02955_gb300 import Context
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("grids chosen for 152 SMs")
+    w = make(nx, nz) if make is moist else W.density_current(nx=nx, nz=nz, nu=nu)
+    ctx = Context(w, dtype=dtype)
+    ctx.use_persistent(mode)
+    info = ctx.info()
+    ctx.close()
+    over = info["tiles_total"] / info["persistent_grid"]  # (that many CTAs, or every tile)
+    assert over == 1.0 or over > 1.15, info
