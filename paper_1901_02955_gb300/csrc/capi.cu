@@ -642,21 +642,32 @@ static void tile_domains(std::vector<DomDev> &doms, const TileVariant &tv, int *
 }
 
 // Default tile shape. The cheaper marching shape (they come first in their set) unless the grid is
-// so small that the one-shot tiles after them finish sooner: one such tile of 256 cells costs an SM 1.55 levels of a
-// marching tile (Jovian 8.6 against 5.5 us, dry 4.3 against 2.8), and no less than 2.4 when the
-// SM has only one or two. Else the first shape (in the order built, the fastest on large grids)
-// whose tiles over all domains fill every SM at least once; else the one with the most tiles.
+// so small that the one-shot tiles after them finish sooner: one such tile of 256 cells costs an SM
+// 1.55 levels of a marching tile (Jovian 8.6 against 5.5 us, dry 4.3 against 2.8), and no less than
+// 2.4 when the SM has only one or two. The FP64 Jovian layouts keep their pipe busy from a tile's
+// first conversion on: a march costs n (cz + 0.7) levels (735 us per level and step: 3440 us for 4
+// levels, 15205 for 20; 0.89 of that beyond one round) and the one-shot tiles 1.12 levels for the mean
+// number of tiles per SM. By the FP32 figures they marched, with the microphysics, 100 x 90 x 100 cells
+// at 26.9 ms per step (one-shot 22.8), 54 x 66 x 120 at 13.9 (11.3) and 54 x 40 x 126 at 8.66 (7.22).
+// Else the first shape (in the order built, the fastest on large grids) whose tiles over all domains
+// fill every SM at least once (counted at heights by evenly spread work); else the one with the most
+// tiles.
 static int default_variant(const snap_ctx *ctx) {
   const int nsm = device_sms();
   if (nsm <= 0) return 0;
   int best = 0, march = -1;
   long long best_tiles = -1;
   double march_cost = 1e300;
+  const bool fp64_moist = !ctx->f32 && ctx->nvap > 0;
   for (int v = 0; v < ctx->ks.nvariants; ++v) {
     const TileVariant &tv = ctx->ks.var[v];
     double cost;
     const int cz = choose_levels(ctx->dom, tv, nsm, &cost, 0, true);
     if (tv.levels == kMarchLevels) {
+      if (fp64_moist) {
+        const long long n = (count_tiles(ctx->dom, tv.tile, cz) + nsm - 1) / nsm;
+        cost = (cz + 0.7) * (n > 1 ? 0.89 * n : 1.0);
+      }
       if (cost < march_cost) {
         march_cost = cost;
         march = v;
@@ -666,7 +677,7 @@ static int default_variant(const snap_ctx *ctx) {
     const long long t = count_tiles(ctx->dom, tv.tile, cz);
     if (march >= 0) {  // this is the first shape after the marching ones
       const long long n = (t + nsm - 1) / nsm;
-      if (march_cost <= std::max(1.55 * n, 2.4)) return march;
+      if (march_cost <= (fp64_moist ? 1.12 * double(t) / nsm : std::max(1.55 * n, 2.4))) return march;
       march = -1;
     }
     if (t >= nsm) return v;
