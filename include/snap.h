@@ -251,14 +251,15 @@ int snap_set_stream(snap_ctx *ctx, void *stream);
 int snap_use_graph(snap_ctx *ctx, int enable);
 
 /* Select one of the tile shapes built for the context's layout (count in
- * snap_info.n_tile_variants; the active one in snap_info.tile_variant). A new context starts
- * on the first shape, in the order built, whose tiles over all domains are at least the
- * device's SM count, else on the shape with the most tiles, so that a small grid still
- * spreads over every SM. In the x-z plane a shape's height is an upper limit: the library takes
- * fewer rows per tile where that spreads a small grid over more SMs (snap_info.tile). In three dimensions (inviscid) the first shape is a march along z: tiles
- * of 32 x 8 columns by a number of levels the library picks for the grid (snap_info.tile); it is
- * the default unless the grid is too small for it. Domains are re-tiled; results do not depend
- * on the shape. */
+ * snap_info.n_tile_variants; the active one in snap_info.tile_variant). In the x-z plane a new
+ * context starts on the first shape, in the order built, whose tiles over all domains are at
+ * least the device's SM count, else on the shape with the most tiles; a shape's height is an
+ * upper limit, and the library takes fewer rows per tile where that spreads a small grid over
+ * more SMs (snap_info.tile). In three dimensions (inviscid) the first shapes are marches along z:
+ * tiles of 32 x 8 columns (variant 0; the FP32 layout of two vapours without microphysics: 32 x
+ * 16, and 32 x 8 as variant 1) by a number of levels the library picks for the grid; the one-shot
+ * shapes (8 x 8 x 4 first) follow, and a cost estimate decides which of the two a new context
+ * starts on. Domains are re-tiled; results do not depend on the shape. */
 int snap_set_tile_variant(snap_ctx *ctx, int variant);
 
 /* Launch mode of a step. 0 (default): three launches per step, one per stage. 1: one
@@ -400,8 +401,8 @@ int snap_probe_fma(int dtype, double *tflops, void *stream);
  * or SNAP_ECUDA (launch failure).
  *
  * snap_check_rcp64: for the n doubles x, y[2i] = the FP64 kernels' reciprocal of x[i]
- * (Newton-Raphson from the approximate hardware reciprocal) and y[2i+1] = 1.0 / x[i] by IEEE
- * division.
+ * (one third-order step from the approximate hardware reciprocal) and y[2i+1] = 1.0 / x[i] by
+ * IEEE division.
  *
  * snap_check_weno: n windows of five values (a, b, c, d, e) = (Q_{c-2} .. Q_{c+2}) of the given
  * dtype, laid out [n][5]; out [n][2] receives the kernels' WENO5 states of Sec. 4.2 (Eq. weno5

@@ -1818,9 +1818,9 @@ extern "C" int snap_use_persistent(snap_ctx *ctx, int enable) {
   return SNAP_OK;
 }
 
-// Times `steps` steps of every tile variant in both launch modes on a copy of the current
+// Times `steps` steps of every tile variant in every launch mode that applies, from the current
 // state, restores the state, and keeps the fastest. best_ms (may be NULL) gets its time per
-// step; choice (may be NULL) gets variant * 2 + persistent.
+// step; choice (may be NULL) gets variant * 3 + launch mode, or -1 for per-class shapes.
 extern "C" int snap_autotune(snap_ctx *ctx, int steps, double *best_ms, int *choice) {
   if (!ctx) return fail(nullptr, SNAP_EINVAL, "snap_autotune: NULL context");
   if (steps < 1) return fail(ctx, SNAP_EINVAL, "snap_autotune: steps < 1");

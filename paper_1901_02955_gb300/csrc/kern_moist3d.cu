@@ -18,7 +18,7 @@ bool find_kernels_moist3d(int f32, int visc, int micro, KernelSet *out) {
   using M2 = MarchT<32, 16, 32, 1>;
   using M64 = MarchT<32, 8, 32, 1>;
   if (visc) return false;
-  if (micro)  // sedimentation and the Kessler scheme compiled in, default tile only
+  if (micro)  // sedimentation and the Kessler scheme compiled in: the march and one one-shot tile
     *out = f32 ? Family<float, L>::set_micro<M, A>() : Family<double, L>::set_micro<M64, A64>();
   else
     *out = f32 ? Family<float, L>::set<false, M2, M, A, B>() : Family<double, L>::set<false, M64, A64>();

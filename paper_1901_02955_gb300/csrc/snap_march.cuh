@@ -201,10 +201,8 @@ __device__ __forceinline__ void march_tiles(const StageArgs &a, const int stage,
           const R pref = P::pf(S, k + 1);
           lmars<R, L>(C, QL, QP, 2, pref, Fn);
           if constexpr (L::MOIST && MICRO) {
-            // no condensate passes a wall
-            if (ph.sediment && !(k + 1 == 0 && S.bc[4] != kBcPeriodic) &&
-                !(k + 1 == nz && S.bc[5] != kBcPeriodic))
-              sediment_flux<R, L>(C, QL, QP, pref, Fn);
+            // no condensate passes a wall (both z sides are)
+            if (ph.sediment && k + 1 != 0 && k + 1 != nz) sediment_flux<R, L>(C, QL, QP, pref, Fn);
           }
         }
         V::store(s_q, tid, NC, QM);

@@ -389,8 +389,8 @@ struct Prof<double> {
 // Conserved -> primitive. y holds the stored state, whose energy entry is rho e - eref with
 // eref = pbar / (gamma_d - 1). x receives (rho, q_i, q_ij, u, [v], w, p - pbar), the total
 // pressure is returned in p_tot and T in T_out. Dry: p - pbar = (gamma_d - 1)(y_E - K) is
-// formed from small numbers. Moist: the inversion U = rho e - K - A, T = U / C_v, p = R_m T
-// runs in FP64.
+// formed from small numbers. Moist, FP64: the inversion U = rho e - K - A, T = U / C_v, p = R_m T;
+// FP32: the same p rewritten as a sum of small numbers.
 template <class R, class L, class DD>
 __device__ __forceinline__ void cons_to_prim(const Phys &ph, const CstT<R> &C, const DD &D,
                                              int k, const R *y, R *x, R &p_tot, R &T_out) {
@@ -644,7 +644,9 @@ struct Wide<double> {
 // T, the heat capacity at constant volume (J/(m^3 K)) and the sum of the gas densities over
 // their molar-mass ratios, from the stored conserved values y (energy as rho e - eref): U =
 // rho e - K - A, T = U / C_v (Eq. energy, App. B). The FP32 kernels sum the kinetic and latent
-// energies (about 1e-4 of U) and the density they need in FP32: their rounding is ~1e-10 of U.
+// energies and the density they need in FP32: these are up to about 1e-3 of U in clear air and 1e-2 in
+// cloud (1e-3 kg/m^3 of water: 2.5e3 of 2e5 J/m^3), so their rounding is 1e-10 to 1e-9 of U, far below
+// the 6e-8 of T by which the FP32 state's densities round C_v.
 template <class R, class L>
 __device__ __forceinline__ void invert_T(const Phys &ph, const CstT<R> &C, const R *y,
                                          typename Wide<R>::T eref, typename Wide<R>::T &T,
@@ -799,7 +801,7 @@ __device__ __forceinline__ int satadj_cell(const Phys &ph, const CstT<R> &C, R *
       // pressure is below saturation, and is then limited to the cloud present. A cloud-free
       // vapour that is subsaturated by more than the FP32 error of this estimate (1e-3
       // relative margin) therefore needs no transfer; if all vapours qualify the cell is left
-      // unchanged, as the FP64 iteration would leave it, after one sweep.
+      // unchanged, as the sweeps would leave it.
       R rho = y[0], K2 = R(0), A = R(0), Cv = y[0];
       bool clear = true;
 #pragma unroll
@@ -1816,11 +1818,9 @@ __device__ __forceinline__ void stage_tiles(const StageArgs &a, const int stage,
           const R pref = fz ? P::pf(D, z0 + iz) : P::pc(D, z0 + iz);
           lmars<R, L>(C, QL, QR, d, pref, F);
           if constexpr (L::MOIST && MICRO) {
-            // no condensate passes a wall
+            // no condensate passes a wall (both z sides are)
             const int kf = z0 + iz;
-            if (fz && ph.sediment && !(kf == 0 && D.bc[4] != kBcPeriodic) &&
-                !(kf == nz && D.bc[5] != kBcPeriodic))
-              sediment_flux<R, L>(C, QL, QR, pref, F);
+            if (fz && ph.sediment && kf != 0 && kf != nz) sediment_flux<R, L>(C, QL, QR, pref, F);
           }
           if constexpr (VISC) {
             const int bi = B::idx(ix + 3, iy + B::HY, iz + 3);  // right cell of the face
@@ -2171,10 +2171,8 @@ __device__ __forceinline__ void plane_tiles(const StageArgs &a, const int stage,
           const R pref = P::pf(Dl, kf);
           lmars<R, L>(C, QL, Qz[m], 2, pref, F);
           if constexpr (L::MOIST && MICRO) {
-            // no condensate passes a wall
-            if (ph.sediment && !(kf == 0 && Dl.bc[4] != kBcPeriodic) &&
-                !(kf == nz && Dl.bc[5] != kBcPeriodic))
-              sediment_flux<R, L>(C, QL, Qz[m], pref, F);
+            // no condensate passes a wall (both z sides are)
+            if (ph.sediment && kf != 0 && kf != nz) sediment_flux<R, L>(C, QL, Qz[m], pref, F);
           }
           if constexpr (VISC)
             viscous_flux<R, L>(C, P::ih(Dl, 2), s_prim, s_th, s_pi, b - BX, b, NB, F);
