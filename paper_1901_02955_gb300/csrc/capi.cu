@@ -8,7 +8,7 @@
 #include <string.h>
 
 #include <algorithm>
-#include <functional>
+#include <map>
 #include <new>
 #include <string>
 #include <vector>
@@ -594,19 +594,20 @@ static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv,
         if (mode == 1) {  // the CTAs take the tiles in turn: the first has one of every round
           c += double((tiles + slots - 1) / slots) * resident * work(cz);
         } else {  // higher top tiles first, each to the SM with the least work so far
-          std::vector<long long> load(nsm, q * work(cz));
-          for (int i = 0; i < int(r); ++i) load[i] += work(cz);
-          const auto later = std::greater<long long>();
-          std::make_heap(load.begin(), load.end(), later);
+          std::map<long long, long long> sms;  // SMs by their work
+          sms[q * work(cz)] = nsm - r;
+          if (r) sms[(q + 1) * work(cz)] = r;
           for (int rows = cz - 1; rows > 0; --rows) {
             c += double(top[rows] / nsm) * work(rows);
-            for (long long i = top[rows] % nsm; i > 0; --i) {
-              std::pop_heap(load.begin(), load.end(), later);
-              load.back() += work(rows);
-              std::push_heap(load.begin(), load.end(), later);
+            for (long long left = top[rows] % nsm; left > 0;) {
+              const auto least = sms.begin();
+              const long long load = least->first, n = std::min(left, least->second);
+              left -= n;
+              if (!(least->second -= n)) sms.erase(least);
+              sms[load + work(rows)] += n;
             }
           }
-          c += double(*std::max_element(load.begin(), load.end()));
+          c += double(sms.rbegin()->first);
         }
       }
       c += 1e-3 * share;  // decides between equals
