@@ -8,7 +8,8 @@
 //
 // Per stage, deterministic (no atomics):
 //   adj_satadj_kernel (moist layouts): one thread per cell maps the adjoint of the adjusted
-//     state to that of the state before the adjustment (temperature inversion in FP64);
+//     state to that of the state before the adjustment (temperature inversion in wide
+//     numbers);
 //   adj_face_kernel (FP32; one launch for the faces of every direction): one thread per face
 //     recomputes the face states from its six-cell stencil, transposes LMARS and WENO5, and
 //     writes the contribution of the face to each of its six stencil cells into
