@@ -938,6 +938,19 @@ static int retile(snap_ctx *ctx, int v, int mode) {
   return SNAP_OK;
 }
 
+// The current shape tiled for a launch mode; nothing to do (nor to wait for) where the heights are the
+// same.
+static int tile_for_mode(snap_ctx *ctx, int mode) {
+  if (ctx->tile_mode == mode) return SNAP_OK;
+  const int nsm = device_sms();
+  double cost;
+  if (choose_levels(ctx->dom, ctx->ks.var[ctx->tv], nsm > 0 ? nsm : 1, &cost, mode) == ctx->dom[0].cz) {
+    ctx->tile_mode = mode;
+    return SNAP_OK;
+  }
+  return retile(ctx, ctx->tv, mode);
+}
+
 // Every domain, and every size class, on tile variant v.
 static int apply_variant(snap_ctx *ctx, int v) {
   for (int &t : ctx->cls_tv) t = v;
@@ -1139,10 +1152,7 @@ static bool resident_possible(snap_ctx *ctx, std::string *why) {
 static int build_resident(snap_ctx *ctx) {
   std::string why;
   if (!resident_possible(ctx, &why)) return fail(ctx, SNAP_ENOTSUP, "snap_use_persistent: " + why);
-  if (ctx->tile_mode != 2) {
-    const int rc = retile(ctx, ctx->tv, 2);
-    if (rc) return rc;
-  }
+  if (const int rc = tile_for_mode(ctx, 2)) return rc;
   const int *shape = ctx->ks.var[ctx->tv].tile;
   const int nt = ctx->ntiles;
   std::vector<std::vector<int>> dep(nt);
@@ -1807,9 +1817,8 @@ extern "C" int snap_use_persistent(snap_ctx *ctx, int enable) {
   if (enable == 2) {
     const int rc = build_resident(ctx);
     if (rc) return rc;
-  } else if (ctx->tile_mode != enable) {
-    const int rc = retile(ctx, ctx->tv, enable);
-    if (rc) return rc;
+  } else if (const int rc = tile_for_mode(ctx, enable)) {
+    return rc;
   }
   ctx->persistent = enable;
   if (ctx->graph) {
@@ -1854,7 +1863,7 @@ extern "C" int snap_autotune(snap_ctx *ctx, int steps, double *best_ms, int *cho
       if (p == 1 && ctx->grid_persistent <= 0) continue;
       if (p == 2 && !resident_possible(ctx, nullptr)) continue;
       ctx->persistent = p;
-      if (p && (rc = retile(ctx, v, p))) break;
+      if ((rc = tile_for_mode(ctx, p))) break;
       rc = snap_step_async(ctx, 1, 0.0);  // warm-up
       if (rc) break;
       CK(cudaEventRecord(e0, ctx->stream));
