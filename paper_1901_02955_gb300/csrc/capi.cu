@@ -531,23 +531,31 @@ static long long count_tiles(const std::vector<DomDev> &doms, const int *tl, int
 //     two per SM at once, instead of 384) 1.33 -> 1.08 ms per step, dry 190 x 131 x 85 (408 tiles of
 //     22 levels instead of 612 of 16) 0.65 -> 0.47 ms.
 //   x-z tiles: rows are dealt to the SM's four schedulers warp by warp, cz of them along x and
-//     cz + 2 along z, plus about a row's worth of conversions and barriers. Full tiles come
+//     cz + 2 along z, plus about a row's worth of conversions and barriers. In FP64, where the pipe is
+//     full however the rows fall, half a unit per row of 32 cells and 1.85, and about 1 more for a second
+//     round of the CTA's threads (one tile per SM, dry 70, 95, 144, 201, 307 and 351 us per step for 2, 4,
+//     8, 12, 18 and 22 rows at 25 us a unit; one vapour 133, 174, 225, 338, 365, 406 and 455 us for 2, 4,
+//     6, 8, 10, 12 and 14 rows at 46 us), 0.3 of it once per SM. Full tiles come
 //     first, the ragged top ones fill the SMs that a last round of full ones leaves idle. On a
 //     grid that fills the SMs this keeps the shape's full height; a small grid gets lower tiles
 //     on more SMs: 128 x 128 cells in FP64 (128 tiles of 4 rows instead of 40 of 14) 233 -> 95 us
 //     per step, the Bryan bubble 200 x 100 in FP64 864 -> 405 us, one moist bubble of 61 x 47 cells in
 //     FP32 29 -> 20 us.
-//     The top tiles' work spreads evenly over the SMs while every tile is co-resident, and about so
-//     over many rounds of several tiles per SM at once. Between one and two rounds, and where an SM
-//     holds one tile, a tile beyond the round waits for another to end and counts whole. Spread
+//     The top tiles' work spreads evenly over the SMs while every tile is co-resident, and the work of
+//     all tiles does over many rounds of several tiles per SM at once. Just beyond one round, and where
+//     an SM holds one tile, a tile beyond the round waits for another to end and counts whole. Spread
 //     evenly there too, a few tiles spilt into another round: 446 x 108 moist FP64 (154 tiles of 10
 //     rows on 152 SMs; whole: 126 of 12) 668 -> 406 us per step, 768 x 256 dry FP32 (312 of 10 on 304
 //     places; 264 of 12) 35 -> 29 us, 628 x 229 moist FP32 (460 of 10 on 456; 400 of 12) 52 -> 41 us;
-//     at full height 535, 37 and 47 us with the kernels of before the lower tiles.
+//     at full height 535, 37 and 47 us with the kernels of before the lower tiles. Over 350 FP64 grids
+//     of 40 x 40 to 1100 x 520 cells this takes 0.94 of the time of the tilings by evenly spread work (at
+//     worst 1.06), over as many FP32 ones 1.00.
 //   One-shot 3-D tiles: their own height.
 // mode: the launch mode the tiling is for (snap_use_persistent). even: spread the top tiles' work
 // evenly whatever their number.
-//   2, the resident step: one tile per SM where that is possible, else as many as are co-resident.
+//   2, the resident step: no more tiles than are co-resident; in FP64, and of a shape of which an SM
+//   holds one, no more than one per SM where that is possible (one vapour, 346 x 162 cells: two per SM on
+//   two SMs 859 us per step, one 467).
 static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv, int nsm,
                          double *cost, int mode = 0, bool even = false) {
   int nzmax = 0, best = tv.tile[2];
@@ -555,14 +563,23 @@ static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv,
   if (tv.levels == kFixedLevels) return best;
   for (const DomDev &D : doms) nzmax = D.nz > nzmax ? D.nz : nzmax;
   const bool march = tv.levels == kMarchLevels;
-  const int resident = std::max(1, tv.max_resident_blocks() / nsm);
+  // (two FP64 tiles share one pipe: an SM works on one at a time)
+  const int resident = tv.fp64 ? 1 : std::max(1, tv.max_resident_blocks() / nsm);
   long long cap = 0;  // most tiles (0: any number)
   if (mode == 2) {
     cap = std::max(0, tv.max_resident_tiles());
-    if (count_tiles(doms, tv.tile, tv.tile[2]) <= nsm) cap = std::min<long long>(cap, nsm);
+    if (resident == 1 && count_tiles(doms, tv.tile, tv.tile[2]) <= nsm) cap = std::min<long long>(cap, nsm);
   }
+  const int round = tv.threads / tv.tile[0];  // rows a CTA takes at once
   const auto quarter = [&](int rows) { return (rows * tv.tile[0] + 127) / 128; };
-  const auto work = [&](int rows) { return quarter(rows) + quarter(rows + 2) + 1; };
+  const auto work = [&](int rows) {
+    if (tv.fp64) return rows * tv.tile[0] / 64.0 + 1.85 + (rows + 2 > round ? 1.0 : 0.0);
+    return double(quarter(rows) + quarter(rows + 2) + 1);
+  };
+  // the same on an SM that has had load before: what a launch costs by itself is in every first tile
+  const auto after = [&](double load, int rows) {
+    return load + work(rows) - (tv.fp64 && load > 0.0 ? 0.3 : 0.0);
+  };
   for (int cz = tv.tile[2]; cz >= (march ? 4 : 1); --cz) {
     if (cz >= 2 * nzmax) continue;
     const long long tiles = count_tiles(doms, tv.tile, cz);
@@ -586,29 +603,43 @@ static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv,
       double ragged = 0.0;  // work of the top tiles
       for (int rows = 1; rows < cz; ++rows) ragged += double(top[rows]) * work(rows);
       const double idle = r ? double(nsm - r) * work(cz) : 0.0;
-      c = double(q + (r ? 1 : 0)) * work(cz) + (ragged > idle ? (ragged - idle) / nsm + 1.0 : 0.0);
+      c = (q + (r ? 1 : 0)) * work(cz) + (ragged > idle ? (ragged - idle) / nsm + 1.0 : 0.0);
       const long long slots = (long long)resident * nsm;
       const double share = c;
-      if (!even && tiles > slots && (resident == 1 || tiles < 2 * slots)) {
+      const bool beyond = tiles > slots && (resident == 1 || 4 * tiles < 5 * slots);
+      const bool doubled = mode == 1 && tiles > nsm && 10 * tiles < 11 * nsm;
+      if (!even && mode == 1 && tiles > slots) {
+        // the CTAs take the tiles in turn: the first has one of every round
+        c = ((tiles + slots - 1) / slots) * resident * work(cz);
+      } else if (!even && tiles >= 2 * slots && resident > 1) {
+        c = (full * work(cz) + ragged) / nsm + 0.5 * work(cz);
+      } else if (!even && doubled && !beyond) {
+        // the last tiles of the queue, the top ones, join full ones on the first SMs
+        int rows = 1;
+        while (rows < cz && !top[rows]) ++rows;
+        c = work(cz) + work(rows);
+      } else if (!even && beyond) {
+        // higher top tiles first, each to the SM with the least work so far
+        std::map<double, long long> sms;  // SMs by their work
+        double each = 0.0;
+        for (long long i = 0; i < q; ++i) each = after(each, cz);
+        sms[each] = nsm - r;
+        if (r) sms[after(each, cz)] = r;
         c = 0.0;
-        if (mode == 1) {  // the CTAs take the tiles in turn: the first has one of every round
-          c += double((tiles + slots - 1) / slots) * resident * work(cz);
-        } else {  // higher top tiles first, each to the SM with the least work so far
-          std::map<long long, long long> sms;  // SMs by their work
-          sms[q * work(cz)] = nsm - r;
-          if (r) sms[(q + 1) * work(cz)] = r;
-          for (int rows = cz - 1; rows > 0; --rows) {
-            c += double(top[rows] / nsm) * work(rows);
-            for (long long left = top[rows] % nsm; left > 0;) {
-              const auto least = sms.begin();
-              const long long load = least->first, n = std::min(left, least->second);
-              left -= n;
-              if (!(least->second -= n)) sms.erase(least);
-              sms[load + work(rows)] += n;
-            }
+        for (int rows = cz - 1; rows > 0; --rows) {
+          c += (top[rows] / nsm) * work(rows);
+          for (long long left = top[rows] % nsm; left > 0;) {
+            const auto least = sms.begin();
+            const double load = least->first;
+            const long long n = std::min(left, least->second);
+            left -= n;
+            if (!(least->second -= n)) sms.erase(least);
+            sms[after(load, rows)] += n;
           }
-          c += double(sms.rbegin()->first);
         }
+        c += sms.rbegin()->first;
+        // a few tiles beyond the round only for more than this estimate's own error (about 4 %)
+        if (tiles > slots && 20 * tiles <= 23 * slots) c *= 1.045;
       }
       c += 1e-3 * share;  // decides between equals
     }
@@ -650,20 +681,28 @@ static void tile_domains(std::vector<DomDev> &doms, const TileVariant &tv, int *
 // levels, 15205 for 20; 0.89 of that beyond one round) and the one-shot tiles 1.12 levels for the mean
 // number of tiles per SM. By the FP32 figures they marched, with the microphysics, 100 x 90 x 100 cells
 // at 26.9 ms per step (one-shot 22.8), 54 x 66 x 120 at 13.9 (11.3) and 54 x 40 x 126 at 8.66 (7.22).
-// Else the first shape (in the order built, the fastest on large grids) whose tiles over all domains
-// fill every SM at least once (counted at heights by evenly spread work); else the one with the most
-// tiles.
+// Else in FP64 the cheapest shape, in FP32 the first (in the order built, the fastest on large grids)
+// whose tiles over all domains fill every SM at least once (counted at heights by evenly spread work),
+// else the one with the most tiles.
 static int default_variant(const snap_ctx *ctx) {
   const int nsm = device_sms();
   if (nsm <= 0) return 0;
   int best = 0, march = -1;
   long long best_tiles = -1;
-  double march_cost = 1e300;
+  double march_cost = 1e300, plane_cost = 1e300;
   const bool fp64_moist = !ctx->f32 && ctx->nvap > 0;
   for (int v = 0; v < ctx->ks.nvariants; ++v) {
     const TileVariant &tv = ctx->ks.var[v];
     double cost;
-    const int cz = choose_levels(ctx->dom, tv, nsm, &cost, 0, true);
+    const bool by_cost = tv.levels == kPlaneLevels && tv.fp64;
+    const int cz = choose_levels(ctx->dom, tv, nsm, &cost, 0, !by_cost);
+    if (by_cost) {
+      if (cost < plane_cost) {
+        plane_cost = cost;
+        best = v;
+      }
+      continue;
+    }
     if (tv.levels == kMarchLevels) {
       if (fp64_moist) {
         const long long n = (count_tiles(ctx->dom, tv.tile, cz) + nsm - 1) / nsm;

@@ -140,6 +140,7 @@ enum LevelChoice : int { kFixedLevels = 0, kMarchLevels = 1, kPlaneLevels = 2 };
 struct TileVariant {
   int tile[3];               // tile[2]: the most levels a tile may have
   int levels;                // how the levels per tile are chosen (LevelChoice)
+  int fp64;                  // 1: FP64 kernels
   int threads;
   size_t smem_stage;
   cudaError_t (*stage)(const StageArgs &, int grid, cudaStream_t);

@@ -137,8 +137,8 @@ __device__ __forceinline__ const CstT<double> &cst<double>(const StageArgs &a) {
 
 // Tile shape: TX x TY x TZ owned cells per CTA of NT threads (TY = 1 in the x-z plane).
 // MINB: CTAs per SM the kernel is compiled for (second __launch_bounds__ argument), which caps
-// its registers; 0 leaves the register count to the compiler. RESB: the same for the resident step,
-// which takes no grid of more tiles than are co-resident.
+// its registers; 0 leaves the register count to the compiler. RESB: the same for the resident step on
+// grids of more tiles than SMs (it takes no grid of more tiles than are co-resident).
 template <int TX_, int TY_, int TZ_, int NT_ = 256, int MINB_ = 0, int RESB_ = MINB_>
 struct TileT {
   static constexpr int TX = TX_, TY = TY_, TZ = TZ_, NT = NT_, MINB = MINB_, RESB = RESB_;
@@ -2318,8 +2318,8 @@ __global__ void __launch_bounds__(T::NT, T::MINB) step_kernel(const StageArgs a)
 // set to 3 seq + s + 1 once the tile's stage-s output is in memory (seq counts the launches) --
 // instead of a grid barrier or a new launch. Waits are bounded like the grid barrier's. The
 // last CTA to finish moves each domain's next CFL rate into place and advances seq.
-template <class R, class L, bool VISC, class T, bool MICRO>
-__global__ void __launch_bounds__(T::NT, T::RESB) resident_step_kernel(const StageArgs a) {
+template <class R, class L, bool VISC, class T, bool MICRO, int MINB>
+__global__ void __launch_bounds__(T::NT, MINB) resident_step_kernel(const StageArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned int s_seq;
   R ys[kept_cells<R, L, VISC, T>()][L::NV];
@@ -2528,14 +2528,19 @@ __global__ void __launch_bounds__(256) satadj_kernel(const StageArgs a, int dm, 
 template <class R, class L, bool VISC, class T, bool MICRO = false>
 struct Variant {
   static constexpr size_t kSmem = stage_smem<R, L, VISC, T>();
+  // the resident step as compiled for its most tiles per SM, and for one (the same but for FP64 with
+  // one vapour)
+  static constexpr auto kResident = &resident_step_kernel<R, L, VISC, T, MICRO, T::RESB>;
+  static constexpr auto kOnePerSm = &resident_step_kernel<R, L, VISC, T, MICRO, T::MINB>;
   static cudaError_t prepare() {
     cudaError_t e = cudaFuncSetAttribute(stage_kernel<R, L, VISC, T, MICRO>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          int(kSmem));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(resident_step_kernel<R, L, VISC, T, MICRO>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
-    if (e != cudaSuccess) return e;
+    for (const auto k : {kResident, kOnePerSm}) {
+      e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
+      if (e != cudaSuccess) return e;
+    }
     return cudaFuncSetAttribute(step_kernel<R, L, VISC, T, MICRO>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, int(kSmem));
   }
@@ -2544,12 +2549,17 @@ struct Variant {
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
       return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &per, resident_step_kernel<R, L, VISC, T, MICRO>, T::NT, kSmem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kResident, T::NT, kSmem) != cudaSuccess)
       return 0;
     return per * nsm;
   }
   static cudaError_t resident(const StageArgs &a, int grid, cudaStream_t s) {
+    int dev = 0, nsm = 0;
+    if (kResident != kOnePerSm) {
+      cudaError_t e = cudaGetDevice(&dev);
+      if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+      if (e != cudaSuccess) return e;
+    }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(T::NT);
@@ -2560,7 +2570,7 @@ struct Variant {
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, resident_step_kernel<R, L, VISC, T, MICRO>, a);
+    return cudaLaunchKernelEx(&cfg, grid <= nsm ? kOnePerSm : kResident, a);
   }
   static cudaError_t stage(const StageArgs &a, int grid, cudaStream_t s) {
     stage_kernel<R, L, VISC, T, MICRO><<<grid, T::NT, kSmem, s>>>(a);
@@ -2595,6 +2605,7 @@ struct Variant {
     v.tile[1] = T::TY;
     v.tile[2] = T::TZ;
     v.levels = T::MARCH ? kMarchLevels : (L::D3 ? kFixedLevels : kPlaneLevels);
+    v.fp64 = sizeof(R) == 8;
     v.threads = T::NT;
     v.smem_stage = kSmem;
     v.stage = &stage;
