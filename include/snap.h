@@ -254,8 +254,9 @@ int snap_use_graph(snap_ctx *ctx, int enable);
  * snap_info.n_tile_variants; the active one in snap_info.tile_variant). In the x-z plane a new
  * context starts on the first shape, in the order built, whose tiles over all domains are at
  * least the device's SM count, else on the shape with the most tiles (in FP64 on the shape the
- * library's estimate finds cheapest, as a rule the first); a shape's height is an upper limit, and the library takes fewer rows per tile where that spreads a small grid over
- * more SMs (snap_info.tile). In three dimensions (inviscid) the first shapes are marches along z:
+ * library's estimate finds cheapest, as a rule the first); a shape's height is an upper limit,
+ * and the library takes fewer rows per tile where that spreads a small grid over more SMs
+ * (snap_info.tile). In three dimensions (inviscid) the first shapes are marches along z:
  * tiles of 32 x 8 columns (variant 0; the FP32 layout of two vapours without microphysics: 32 x
  * 16, and 32 x 8 as variant 1) by a number of levels the library picks for the grid; the one-shot
  * shapes (8 x 8 x 4 first) follow, and a cost estimate decides which of the two a new context
