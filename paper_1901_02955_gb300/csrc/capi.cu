@@ -535,7 +535,7 @@ static long long count_tiles(const std::vector<DomDev> &doms, const int *tl, int
 //     full however the rows fall, half a unit per row of 32 cells and 1.85, and about 1 more for a second
 //     round of the CTA's threads (one tile per SM, dry 70, 95, 144, 201, 307 and 351 us per step for 2, 4,
 //     8, 12, 18 and 22 rows at 25 us a unit; one vapour 133, 174, 225, 338, 365, 406 and 455 us for 2, 4,
-//     6, 8, 10, 12 and 14 rows at 46 us), 0.3 of it once per SM. Full tiles come
+//     6, 8, 10, 12 and 14 rows at 46 us; one row takes as long as two), 0.3 of it once per SM. Full tiles come
 //     first, the ragged top ones fill the SMs that a last round of full ones leaves idle. On a
 //     grid that fills the SMs this keeps the shape's full height; a small grid gets lower tiles
 //     on more SMs: 128 x 128 cells in FP64 (128 tiles of 4 rows instead of 40 of 14) 233 -> 95 us
@@ -573,7 +573,8 @@ static int choose_levels(const std::vector<DomDev> &doms, const TileVariant &tv,
   const int round = tv.threads / tv.tile[0];  // rows a CTA takes at once
   const auto quarter = [&](int rows) { return (rows * tv.tile[0] + 127) / 128; };
   const auto work = [&](int rows) {
-    if (tv.fp64) return rows * tv.tile[0] / 64.0 + 1.85 + (rows + 2 > round ? 1.0 : 0.0);
+    if (tv.fp64)
+      return std::max(rows, 2) * tv.tile[0] / 64.0 + 1.85 + (rows + 2 > round ? 1.0 : 0.0);
     return double(quarter(rows) + quarter(rows + 2) + 1);
   };
   // the same on an SM that has had load before: what a launch costs by itself is in every first tile
